@@ -127,9 +127,9 @@ typedef struct dao_options {
                                 * iterate together (bounded grid barriers); 0, or where a cooperative
                                 * launch is not available: one launch per evaluation kernel */
     int32_t mlc_constraint;    /* DAO_MLC_* of the pricing (default DAO_MLC_CONSECUTIVE) */
-    int32_t master_blocks;     /* blocks of the persistent master solve; 0 (default): two per SM, the whole
-                                * GPU; fewer (raised to the least whose per-block working set fits shared
-                                * memory) leave room for other plans' solves to run side by side */
+    int32_t master_blocks;     /* blocks of the persistent master solve; 0 (default): one per SM, or fewer
+                                * where they give every warp its voxels; n > 0: n blocks (at most one per SM),
+                                * which leaves room for other plans' solves to run side by side */
     int32_t dt_threads;        /* threads per beamlet row of the transposed SpMV: 0 (default: 64, or the
                                 * autotuner's choice), 64, 128 or 256 */
     int32_t dt_map;            /* form of the transposed SpMV: 0 (default: DAO_DT_CONSECUTIVE, or the
@@ -443,20 +443,19 @@ dao_status dao_batch_solve(dao_ctx* const* ctxs, int32_t n, int32_t n_apertures,
 
 /* Column generation for n independent contexts with one persistent master
  * launch per round for all of them: the plans' master solves run side by side
- * in one cooperative kernel, each on its own group of blocks (two blocks per SM
- * shared out evenly; each group with its own grid barrier, solver state and
+ * in one cooperative kernel (two, when there are more plans than SMs), each on
+ * its own group of blocks (one block per SM shared out evenly; each group with its own grid barrier, solver state and
  * stopping), while every plan's D^T kernel and beam decision with the new
  * column run on its own stream before it.  The rounds are captured once into
  * a CUDA graph for the list of contexts and the round count, kept for the
  * next call with the same list (at most four such graphs; a graph goes with
  * its contexts' dao_destroy).  Arguments and results as dao_batch_solve; a
  * plan's results are those of solving it alone with a persistent master of
- * the same group size.  DAO_EINVAL when two blocks per SM do not give every
- * plan a block (n > 2 x SMs).  Synchronous. */
+ * the same group size.  DAO_EINVAL when n > 2 x SMs.  Synchronous. */
 dao_status dao_batch_solve_persistent(dao_ctx* const* ctxs, int32_t n, int32_t n_apertures, int32_t* n_done,
                                       double* traces, int32_t* status);
 
-/* Blocks per plan of dao_batch_solve_persistent for n plans on device `device` (0 when n plans do not fit one launch): a plan
+/* Blocks per plan of dao_batch_solve_persistent for n plans on device `device` (0 when n > 2 x SMs): a plan
  * created with this master_blocks solves alone exactly as it does in the
  * batch. */
 int32_t dao_batch_group_size(int32_t n, int32_t device);

@@ -94,7 +94,7 @@ struct dao_ctx {
     // column-generation state
     int K = 0, K_cap = 0, ld = 0;
     int async_K0 = 0, async_K1 = 0;  // rounds launched by solve_async_begin
-    float* slab = nullptr;           // K_cap x ld, column k = dose of aperture k (Eq. 2)
+    float* slab = nullptr;           // column k = dose of aperture k (Eq. 2), four columns interleaved (slab_column)
     std::vector<int> ap_beam_h, ap_lr_h;
     int* ap_beam = nullptr;
     int* ap_lr = nullptr;            // K_cap x 2*max_rows
@@ -405,6 +405,7 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
         free_temps();
         return fail(DAO_EINVAL, "voxel structure label out of range at voxel " + std::to_string(V - chk.bad_label));
     }
+    c->mb.nonneg = chk.negative == 0;
     const int64_t padded = chk.padded;
     if (padded >= (int64_t)1 << 31) {
         free_temps();
@@ -604,8 +605,9 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
     return DAO_OK;
 }
 
-// 2-D tensor maps over the column-major slab (column k = aperture k, stride
-// ld floats): box = (MASTER_TILE voxels, KP columns), one map per KP.
+// 2-D tensor maps over the slab (a row per group of four columns: ld voxels of 16
+// bytes) in 8-byte elements: box = (half of MASTER_TILE voxels, KP / 4 groups), one
+// map per KP.
 dao_status make_tensor_maps(dao_ctx* c) {
     typedef CUresult (*encode_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -617,22 +619,12 @@ dao_status make_tensor_maps(dao_ctx* c) {
     encode_fn encode = reinterpret_cast<encode_fn>(fn);
     std::memset(c->mb.tmap, 0, sizeof(c->mb.tmap));
     for (int kp = 4; kp <= KMAX; kp += 4) {
-        const cuuint64_t dims[2] = {(cuuint64_t)c->ld, (cuuint64_t)KMAX};
-        const cuuint64_t strides[1] = {(cuuint64_t)c->ld * sizeof(float)};
-        const cuuint32_t box[2] = {(cuuint32_t)MASTER_TILE, (cuuint32_t)kp};
+        const cuuint64_t dims[2] = {(cuuint64_t)c->ld * 2, (cuuint64_t)KMAX / 4};
+        const cuuint64_t strides[1] = {(cuuint64_t)c->ld * 4 * sizeof(float)};
+        const cuuint32_t box[2] = {(cuuint32_t)MASTER_TILE, (cuuint32_t)kp / 4};
         const cuuint32_t estr[2] = {1, 1};
-        CUresult r = encode(&c->mb.tmap[kp / 4], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, c->slab, dims, strides, box, estr,
+        CUresult r = encode(&c->mb.tmap[kp / 4], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, c->slab, dims, strides, box, estr,
                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(DAO_ECUDA, "cuTensorMapEncodeTiled failed with " + std::to_string((int)r));
-    }
-    for (int m = 0; m < 2; ++m) {  // the persistent solve's maps: boxes of 128 voxels x 16, x 4 columns
-        const cuuint64_t dims[2] = {(cuuint64_t)c->ld, (cuuint64_t)KMAX};
-        const cuuint64_t strides[1] = {(cuuint64_t)c->ld * sizeof(float)};
-        const cuuint32_t box[2] = {128u, m == 0 ? 16u : 4u};
-        const cuuint32_t estr[2] = {1, 1};
-        CUresult r = encode(&c->mb.tmap_p[m], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, c->slab, dims, strides, box, estr,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return fail(DAO_ECUDA, "cuTensorMapEncodeTiled failed with " + std::to_string((int)r));
     }
@@ -862,7 +854,7 @@ dao_status add_column(dao_ctx* c, int beam, const int32_t* lr, float* out, int s
 
 // Column and table entry of aperture (beam, lr) at pool index K; no master solve.
 dao_status append_aperture(dao_ctx* c, int beam, const int32_t* lr) {
-    DAO_TRY(add_column(c, beam, lr, c->slab + (size_t)c->K * c->ld, 1));
+    DAO_TRY(add_column(c, beam, lr, slab_column(c->slab, c->ld, c->K), SLAB_STRIDE));
     const int stride = 2 * c->max_rows;
     c->ap_beam_h.push_back(beam);
     c->ap_lr_h.resize((size_t)(c->K + 1) * stride, 0);
@@ -2201,10 +2193,9 @@ dao_status build_batch_graph(dao_ctx* const* ctxs, int n, int R, BatchGraph* bg)
     dao_ctx* c0 = ctxs[0];
     bg->device = c0->device;
     bg->GB = master_batch_group(n, c0->num_sms);
-    if (bg->GB < 1) return fail(DAO_EINVAL, "too many plans for one persistent launch (two blocks per SM each)");
+    if (bg->GB < 1) return fail(DAO_EINVAL, "too many plans for the persistent batch (at most two per SM)");
     DAO_CU(cudaStreamCreateWithFlags(&bg->stream, cudaStreamNonBlocking));
     std::vector<MasterTask> tasks(n);
-    int max_V = 0;
     for (int i = 0; i < n; ++i) {
         dao_ctx* c = ctxs[i];
         MasterTask& t = tasks[i];
@@ -2228,11 +2219,9 @@ dao_status build_batch_graph(dao_ctx* const* ctxs, int n, int R, BatchGraph* bg)
         t.z_out = c->z;
         t.pi_out = c->pi;
         t.cg = c->cg;
-        t.tmap[0] = c->mb.tmap_p[0];
-        t.tmap[1] = c->mb.tmap_p[1];
         t.vstate = c->mb.vstate;
         t.H_keep = c->mb.H_keep;
-        max_V = std::max(max_V, c->V);
+        t.nonneg = c->mb.nonneg;
     }
     void* tp = nullptr;
     DAO_CU(pool_alloc(&tp, sizeof(MasterTask) * n, bg->device, bg->stream));
@@ -2278,7 +2267,7 @@ dao_status build_batch_graph(dao_ctx* const* ctxs, int n, int R, BatchGraph* bg)
             check(cudaEventRecord(bg->events[i], cs));
             check(cudaStreamWaitEvent(bg->stream, bg->events[i], 0));
         }
-        check(launch_master_persist_batch(bg->tasks, n, bg->GB, max_V, bg->stream, &nl));
+        check(launch_master_persist_batch(bg->tasks, n, bg->GB, c0->num_sms, bg->stream, &nl));
     }
     cudaGraph_t g = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(bg->stream, &g);

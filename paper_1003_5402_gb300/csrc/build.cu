@@ -266,13 +266,16 @@ __global__ void k_check(const int64_t* __restrict__ rp, const int* __restrict__ 
         const int64_t p0 = rp[j], p1 = rp[j + 1];
         bool ok = p0 >= 0 && p1 >= p0 && p1 <= nnz;
         if (ok) {
-            bool bad = false;
+            bool bad = false, neg = false;
             for (int64_t p = p0 + lane; p < p1; p += 32) {
                 const int c = col[p];
-                bad |= c < 0 || c >= N || !isfinite(val[p]);
+                const float v = val[p];
+                bad |= c < 0 || c >= N || !isfinite(v);
+                neg |= v < 0.f;
                 if (p > p0) bad |= c <= col[p - 1];
             }
             ok = !__any_sync(FULL, bad);
+            if (__any_sync(FULL, neg) && lane == 0) chk->negative = 1;
         }
         if (lane == 0) {
             plen[j] = ok ? (p1 - p0 + pad - 1) / pad * pad : 0;

@@ -31,6 +31,14 @@ constexpr int CMAX = 32;        // beamlets per MLC row (one warp lane each)
 constexpr int MASTER_TILE = 256;  // voxels per tile of the master evaluation (= block size)
 constexpr int KROW = KMAX + 4;    // row stride (floats) of the active-voxel rows (odd float4 count)
 
+// Column k of the aperture slab of column height ld: entry j at
+// slab_column(slab, ld, k)[SLAB_STRIDE * j].  Four columns are interleaved, so that
+// one 16-byte load gives a voxel's doses of a group of four.
+constexpr int SLAB_STRIDE = 4;
+__host__ __device__ inline float* slab_column(float* slab, int ld, int k) {
+    return slab + (size_t)(k / 4) * ld * 4 + k % 4;
+}
+
 // Per-structure objective terms (Eqs. 9-10): a = alpha_s/|v_s| (0 for
 // non-targets), tu = T_s^-, b = beta_s/|v_s|, to = T_s^+.
 struct StructTermsF { float a, tu, b, to; };
@@ -136,6 +144,12 @@ struct MasterDev {
     float Ht[KMAX * KMAX];   // curvature matrix at the trial point (full, symmetric; FP64 sums
                              // rounded once to FP32, the precision of the factorisation)
     float gn[KMAX];       // sum_j |S_jk pi_j| at the trial point: the rounding scale of g_k
+    // persistent solve: the reduced sums as words of 32 bits under the number of
+    // their evaluation (H's lower triangle, row-major; FP64 values in two words)
+    unsigned long long wH[KMAX * KMAX];
+    unsigned long long wg[2 * KMAX];
+    unsigned long long wgn[KMAX];
+    unsigned long long wF[2];
     double F;             // objective at y
     double Ft;            // objective at the trial point
     double alpha;         // step length along d
@@ -152,6 +166,7 @@ struct MasterDev {
     int final_pending;    // the solve stopped at an accepted point other than the last one evaluated
     int inc_G;            // persistent solve: group size whose kept partial H and voxel states are valid (0: none)
     int inc_K;            // the pool size they were kept at
+    unsigned epoch;       // persistent solve: evaluations since the state was cleared
 };
 
 enum { MASTER_RUNNING = 0, MASTER_CONVERGED = 1, MASTER_MAXITER = 2, MASTER_STALLED = 3, MASTER_ERROR = 4 };
@@ -363,9 +378,9 @@ struct MasterBuffers {
     int GP = 0;                 // blocks of the persistent solve (co-resident), 0: not available
     int grid[KMAX + 1] = {};    // blocks of the evaluation kernel for each pool size
     CUtensorMap tmap[KMAX / 4 + 1];  // slab tile maps, indexed by columns / 4
-    CUtensorMap tmap_p[2];           // slab maps of the persistent solve: boxes of 128 voxels x 16, x 4 columns
     uint8_t* vstate = nullptr;       // [V] persistent solve: each voxel's curvature state at the last evaluation
     float* H_keep = nullptr;         // [GH][KMAX*(KMAX+1)/2] persistent solve: each block's kept partial H
+    int nonneg = 0;                  // no entry of D is negative
 };
 enum { PASS_EVAL = 0, PASS_FINAL = 1, PASS_TIMING = 2 };
 __host__ __device__ int master_kw(int K);
@@ -409,11 +424,12 @@ void pinned_release(void* p, size_t bytes);
 cudaError_t release_cached_memory(int device);
 
 // Result of the device-side input checks: the first bad CSR row and the first
-// bad structure label as V - index (0: none), the padded entry count of D and
-// the voxels of each structure.
+// bad structure label as V - index (0: none), whether an entry is negative, the
+// padded entry count of D and the voxels of each structure.
 struct BuildCheck {
     int bad_row;
     int bad_label;
+    int negative;        // some entry is below 0
     long long padded;
     int count[SMAX];
 };
@@ -458,7 +474,6 @@ cudaError_t build_transpose_place(int prec, const int64_t* rp, const int* col, c
 // the slab and its partial arrays (stride GS), the objective terms, the
 // round's skip flag and outputs, and the device-side round state (pool size).
 struct MasterTask {
-    CUtensorMap tmap[2];  // the slab in boxes of 128 voxels x 16, x 4 columns (MasterBuffers::tmap_p)
     const float* slab;
     int ld, V, GS, S, max_iter;
     MasterDev* st;
@@ -476,23 +491,23 @@ struct MasterTask {
     CGDev* cg;
     uint8_t* vstate;      // MasterBuffers::vstate
     float* H_keep;        // MasterBuffers::H_keep
+    int nonneg;           // MasterBuffers::nonneg
 };
-// Several plans' master solves in one cooperative launch, GB blocks each
-// (master_batch_group: the most for n_tasks plans with two blocks per SM);
-// tasks in device memory; max_V the largest voxel count.
+// Several plans' master solves in one cooperative launch (two when there are
+// more plans than SMs), GB blocks each (master_batch_group: the most for n_tasks
+// plans with one block per SM); tasks in device memory.
 int master_batch_group(int n_tasks, int num_sms);
-cudaError_t launch_master_persist_batch(const MasterTask* tasks, int n_tasks, int GB, int max_V, cudaStream_t stream,
-                                        int* launches);
+cudaError_t launch_master_persist_batch(const MasterTask* tasks, int n_tasks, int GB, int num_sms,
+                                        cudaStream_t stream, int* launches);
 
-// The whole master solve as one cooperative launch (GP blocks), after
-// launch_master_init; dynamic shared memory per master_persist_smem.
-size_t master_persist_smem(int V, int G);
 // Diagnostic: a cooperative launch whose block `absent` never arrives at the
 // grid barrier; out[0] counts the blocks whose bounded wait gave up, out[1]
 // those that passed.
 cudaError_t launch_barrier_check(GridBar* gb, int blocks, int absent, int* out, cudaStream_t stream);
+// The whole master solve as one cooperative launch of GP blocks
+// (master_persist_grid).
 int master_persist_grid(int V, int num_sms, int want = 0);
-// Includes k_master_init's warm start, writes z and pi of the final point, and
+// launch_master_persist includes k_master_init's warm start, writes z and pi of the final point, and
 // (cg != nullptr) the round's record.  K = 0: the pool size is read from
 // cg->K when the kernel runs.
 cudaError_t launch_master_persist(const MasterBuffers& mb, const float* slab, int ld, int V, int K,

@@ -1,7 +1,9 @@
 // Master problem of column-generation DAO (arXiv:1003.5402, Sec. 2.2-2.3):
 // min_y F(S y) subject to y >= 0 over the current aperture pool, where column k
-// of the slab S (V x K, FP32, column-major with stride ld) is the aperture dose
-// D_kj of Eq. 2.
+// of the slab S (V x K, FP32) is the aperture dose D_kj of Eq. 2.  The slab is
+// stored by groups of four columns, the four doses of a voxel together (entry
+// (j, k) at ((k / 4) ld + j) 4 + k mod 4): one 16-byte load gives a voxel's
+// doses of a group, and a warp's 32 voxels are 512 consecutive bytes.
 //
 // The paper uses gradient projection and gives no step or stopping rule.  This
 // is a scaled gradient projection, the projected Newton method of Bertsekas
@@ -88,7 +90,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
 }
 
 // 2-D tiled bulk copy of box (x, y) of the tensor map into shared memory.
-__device__ __forceinline__ void tma_load_2d(float* dst, const CUtensorMap* map, int x, int y,
+__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y,
                                             unsigned long long* bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::"r"(
@@ -173,9 +175,8 @@ __global__ void k_cg_record(const MasterDev* __restrict__ st, CGDev* __restrict_
 }
 
 // ---- evaluation: one slab tile per iteration --------------------------------
-// The slab is column-major (column k = the doses of aperture k over all voxels,
-// stride ld); a tile is the box of KP columns x TILE voxels, landing in shared
-// memory as [KP][TILE].
+// A tile is TILE voxels x KP columns of the slab: two boxes of 128 voxels x KP / 4
+// groups of columns, each landing in shared memory as [KP / 4][128][4].
 __global__ void __launch_bounds__(TILE, 3) k_master_eval(const __grid_constant__ CUtensorMap tmap, int V, int K,
                                                          int KP, MasterDev* __restrict__ st,
                                                          float* __restrict__ act_rows, float2* __restrict__ act_hp,
@@ -187,7 +188,7 @@ __global__ void __launch_bounds__(TILE, 3) k_master_eval(const __grid_constant__
     if (skip != nullptr && *skip) return;
     if (mode == PASS_EVAL && st->done) return;
     const bool final_pass = mode == PASS_FINAL;
-    extern __shared__ __align__(128) float As[];  // [KP][TILE]
+    extern __shared__ __align__(128) float4 As[];  // [2][KP / 4][TILE / 2]
     __shared__ __align__(8) unsigned long long bar;
     __shared__ float s_yh[KMAX], s_yl[KMAX];
     __shared__ int s_wcount[TILE / 32];
@@ -208,11 +209,13 @@ __global__ void __launch_bounds__(TILE, 3) k_master_eval(const __grid_constant__
     unsigned parity = 0;
     bool lost = false;
     const int n_tiles = (V + TILE - 1) / TILE;
+    const float4* av = As + (tid / (TILE / 2)) * (KP / 4) * (TILE / 2) + tid % (TILE / 2);  // this voxel, group 0
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         __syncthreads();  // every thread is done with the previous tile's buffers
         if (tid == 0 && KP > 0) {
             mbar_expect_tx(&bar, (unsigned)(TILE * KP * sizeof(float)));
-            tma_load_2d(As, &tmap, tile * TILE, 0, &bar);
+            tma_load_2d(As, &tmap, tile * TILE * 2, 0, &bar);  // (8-byte elements)
+            tma_load_2d(As + (KP / 4) * (TILE / 2), &tmap, tile * TILE * 2 + TILE, 0, &bar);
         }
         if (KP > 0) {
             if (!mbar_wait(&bar, parity)) {
@@ -225,10 +228,11 @@ __global__ void __launch_bounds__(TILE, 3) k_master_eval(const __grid_constant__
         // ---- compensated z from this voxel's column of the tile, four chains
         float sc[4] = {0.f, 0.f, 0.f, 0.f}, cc[4] = {0.f, 0.f, 0.f, 0.f};
         for (int k = 0; k < KP; k += 4) {  // doses of columns K..KP-1 meet y = 0
-            dot2_step(sc[0], cc[0], As[k * TILE + tid], s_yh[k], s_yl[k]);
-            dot2_step(sc[1], cc[1], As[(k + 1) * TILE + tid], s_yh[k + 1], s_yl[k + 1]);
-            dot2_step(sc[2], cc[2], As[(k + 2) * TILE + tid], s_yh[k + 2], s_yl[k + 2]);
-            dot2_step(sc[3], cc[3], As[(k + 3) * TILE + tid], s_yh[k + 3], s_yl[k + 3]);
+            const float4 a = av[(k / 4) * (TILE / 2)];
+            dot2_step(sc[0], cc[0], a.x, s_yh[k], s_yl[k]);
+            dot2_step(sc[1], cc[1], a.y, s_yh[k + 1], s_yl[k + 1]);
+            dot2_step(sc[2], cc[2], a.z, s_yh[k + 2], s_yl[k + 2]);
+            dot2_step(sc[3], cc[3], a.w, s_yh[k + 3], s_yl[k + 3]);
         }
         float s = sc[0], c = cc[0];
 #pragma unroll
@@ -269,9 +273,7 @@ __global__ void __launch_bounds__(TILE, 3) k_master_eval(const __grid_constant__
         if (act) {
             const size_t slot = (size_t)tile * TILE + base + __popc(bal & ((1u << lane) - 1u));
             float4* dst = reinterpret_cast<float4*>(act_rows + slot * KROW);
-            for (int k = 0; k < KP; k += 4)
-                dst[k / 4] = make_float4(As[k * TILE + tid], As[(k + 1) * TILE + tid], As[(k + 2) * TILE + tid],
-                                         As[(k + 3) * TILE + tid]);
+            for (int g = 0; g < KP / 4; ++g) dst[g] = av[g * (TILE / 2)];
             act_hp[slot] = make_float2(h, p);
         }
         if (tid == 0) act_count[tile] = n_act;
@@ -527,133 +529,322 @@ __device__ __forceinline__ void master_reduce_part(const float* __restrict__ H_p
     }
 }
 
-// Block-wide reductions over STEP_T threads with a fixed order.
-constexpr int STEP_T = 256;
-constexpr int STEP_W = STEP_T / 32;
-// Thread roles in a panel of the step's factorisation: warps 0-5 update the
-// rows of the trailing tiles, warp 6 writes the panel's final columns and
-// pivots, warp 7 eliminates the right-hand side.
-constexpr int FACT_TILE_T = 192, FACT_COLW = 192, FACT_RHSW = 224;
-static_assert(STEP_T == 256 && KMAX == 64, "the step kernel maps a 16 x 16 thread grid onto 64 x 64 entries");
-
-// Maximum over the warp of non-negative doubles: their IEEE bit patterns order
-// like their values, so a 64-bit integer maximum is exact and stays off the
-// FP64 pipe (1/64 of the FP32 rate on this part).  A NaN counts as 0, as
-// fmax would skip it.
-__device__ __forceinline__ long long nonneg_bits(double v) { return __double_as_longlong(v == v ? v : 0.0); }
-__device__ __forceinline__ double warp_max_nonneg(double v) {
-    long long b = nonneg_bits(v);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(FULL, b, o));
-    return __longlong_as_double(b);
+// ---- tagged words ------------------------------------------------------------
+// The persistent solve's reduced sums as 64-bit words, 32 bits of the value
+// under the evaluation's number: a reader polls the words it needs, so that no
+// barrier (release, counter, poll, then the loads) lies between the reduction and
+// the step.  An aligned 64-bit access is single-copy atomic, so a word with the
+// right number has its value.  Every word of an evaluation is read by every
+// block before it arrives at the next evaluation's barrier, and rewritten only
+// after that barrier.
+__device__ __forceinline__ void word_put(unsigned long long* p, unsigned v, unsigned tag) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(((unsigned long long)tag << 32) | v) : "memory");
+}
+__device__ __forceinline__ unsigned long long word_get(const unsigned long long* p) {
+    unsigned long long w;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+    return w;
+}
+__device__ __forceinline__ void word_put_f64(unsigned long long* p, double v, unsigned tag) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    word_put(p, (unsigned)b, tag);
+    word_put(p + 1, (unsigned)(b >> 32), tag);
+}
+__device__ __forceinline__ double words_f64(unsigned long long lo, unsigned long long hi) {
+    return __longlong_as_double((long long)((hi << 32) | (lo & 0xffffffffull)));
 }
 
-__device__ __forceinline__ float blk_max_f32(float v, float* sw) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(FULL, v, o));
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = v;
-    __syncthreads();
-    float t = sw[0];
-#pragma unroll
-    for (int w = 1; w < STEP_W; ++w) t = fmaxf(t, sw[w]);
-    return t;
-}
-
-
-// One block: thread k < K owns variable k; all threads share the factorisation.
-__device__ __forceinline__ void master_step_body(MasterDev* __restrict__ st, int max_iter, double tol_rel,
-                                                 double sigma) {
-    __shared__ __align__(16) float A[KMAX][KMAX + 4];   // working lower triangle
-    __shared__ __align__(16) float Lw[KMAX][KMAX + 4];  // final panel columns, L_ik d_k
-    __shared__ __align__(16) float u[KMAX];             // right-hand side being eliminated
-    __shared__ __align__(16) float ye[KMAX];            // eliminated right-hand side
-    __shared__ float piv[KMAX];
-    __shared__ float rd[KMAX];
-    __shared__ float rhs[KMAX];
-    __shared__ float sg[KMAX];                          // FP32 gradient at the accepted point
-    __shared__ float swf[STEP_W];
-    __shared__ int fidx[KMAX];
-    __shared__ double sw[STEP_W];
-    __shared__ double sw2[STEP_W];
-    __shared__ double sw3[STEP_W];
-    __shared__ int swi[STEP_W];
-    // every value the step reads is loaded up front (independent loads, one round
-    // trip); gt, gn, Ft and Ht were written by other blocks of this launch and
-    // are read through L2 (__ldcg), never from a possibly stale L1 line
-    const int k = threadIdx.x;
-    const int kk = k < KMAX ? k : KMAX - 1;
-    // (all through L2: a persistent solve runs the step in whichever block
-    // finishes last, so no L1 line of another iteration may be trusted)
-    const int done = __ldcg(&st->done), err = __ldcg(&st->err), K = __ldcg(&st->K), phase = __ldcg(&st->phase);
-    const int iter0 = __ldcg(&st->iter);
-    const double tol0 = __ldcg(&st->tol), F0 = __ldcg(&st->F), Ft = __ldcg(&st->Ft);
-    const double yt_ = __ldcg(&st->yt[kk]), gt_ = __ldcg(&st->gt[kk]), gn_ = (double)__ldcg(&st->gn[kk]);
-    const double y_ = __ldcg(&st->y[kk]), g_ = __ldcg(&st->g[kk]);
-    // the curvature matrix, requested now so that its latency passes behind the
-    // reductions below; stored to shared memory once the free set is known
-    // (entry 256 m + k of the row-major KMAX x KMAX array)
-    float hpre[KMAX * KMAX / STEP_T];
-#pragma unroll
-    for (int m = 0; m < KMAX * KMAX / STEP_T; ++m) hpre[m] = __ldcg(&st->Ht[m * STEP_T + k]);
-    if (done) return;
-    if (err) {  // a tile copy was lost in an evaluation: stop with the last accepted point
-        if (threadIdx.x == 0) {
-            st->status = MASTER_ERROR;
-            st->final_pending = 1;
-            st->done = 1;
+// Reduction of the partial sums of one evaluation (as master_reduce_part) into
+// tagged words.  last_only: only the outputs of variable K - 1 (column K - 1 of H,
+// its g and gn).
+__device__ __forceinline__ void master_reduce_words(const float* __restrict__ H_part,
+                                                    const double* __restrict__ g_part,
+                                                    const float* __restrict__ gn_part,
+                                                    const double* __restrict__ F_part, int GS, int G, int K,
+                                                    MasterDev* st, int bid, bool last_only, unsigned tag) {
+    const int E = K * (K + 1) / 2;
+    const int lane = threadIdx.x & 31;
+    const int n_out = last_only ? K + 2 : E + 2 * K + 1;
+    for (int o_ = (bid * (int)blockDim.x + (int)threadIdx.x) >> 5; o_ < n_out; o_ += (G * (int)blockDim.x) >> 5) {
+        const int o = !last_only ? o_ : o_ < K ? E - K + o_ : o_ == K ? E + K - 1 : E + 2 * K - 1;
+        if (o < E) {  // the factorisation is FP32: so is this sum
+            const float x = warp_sum_f32(lane_sum_strided(H_part + (size_t)o * GS, G, lane));
+            if (lane == 0) {  // o = c (c + 1) / 2 + r, r <= c: row c, column r of the lower triangle
+                int c = (int)((sqrtf(8.f * (float)o + 1.f) - 1.f) * 0.5f);
+                while ((c + 1) * (c + 2) / 2 <= o) ++c;
+                while (c * (c + 1) / 2 > o) --c;
+                word_put(&st->wH[c * KMAX + o - c * (c + 1) / 2], __float_as_uint(x), tag);
+            }
+        } else if (o < E + K) {
+            const double x = warp_sum_f64(lane_sum_strided(g_part + (size_t)(o - E) * GS, G, lane));
+            if (lane == 0) word_put_f64(&st->wg[2 * (o - E)], x, tag);
+        } else if (o < E + 2 * K) {
+            const float x = warp_sum_f32(lane_sum_strided(gn_part + (size_t)(o - E - K) * GS, G, lane));
+            if (lane == 0) word_put(&st->wgn[o - E - K], __float_as_uint(x), tag);
+        } else {
+            const double x = warp_sum_f64(lane_sum_strided(F_part, G, lane));
+            if (lane == 0) word_put_f64(&st->wF[0], x, tag);
         }
-        return;
     }
-    const bool own = k < K;
-    // only the first nw warps hold variables (K <= 64): they alone run the FP64
-    // reductions, which issue at 1/64 of the FP32 rate on this part
-    const int nw = (K + 31) >> 5;
-    const bool vwarp = (k >> 5) < nw;
-    const double yt = own ? yt_ : 0.0, gt = own ? gt_ : 0.0, gn = own ? gn_ : 0.0;
-    const double y = own ? y_ : 0.0, g = own ? g_ : 0.0;
+}
+
+// The step's threads: the first STEP_T of a block that may have more.
+constexpr int STEP_T = 256;
+constexpr int H_LD = KMAX + 4;  // row stride of H in the step's memory
+static_assert(STEP_T == 256 && KMAX == 64, "the step maps a 16 x 16 thread grid onto 64 x 64 entries");
+
+// Barrier of the step's threads.
+__device__ __forceinline__ void step_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
+// The bit pattern of a non-negative double (0 for a NaN, as fmax would skip it).
+// Patterns order like the values, so maxima and comparisons of non-negative
+// doubles stay on the integer pipe: FP64 issues at 1/64 of the FP32 rate on
+// this part, and the step is a chain of them.
+constexpr unsigned long long INF_BITS = 0x7ff0000000000000ull;
+__device__ __forceinline__ unsigned long long raw_bits(double v) { return (unsigned long long)__double_as_longlong(v); }
+__device__ __forceinline__ unsigned long long nonneg_bits(double v) {
+    const unsigned long long b = raw_bits(v);
+    return b <= INF_BITS ? b : 0ull;
+}
+// fmax(v, 0.0) on the bit pattern.
+__device__ __forceinline__ double relu_bits(double v) { return __longlong_as_double((long long)nonneg_bits(v)); }
+// |v| as a bit pattern, 0 for a NaN.
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+    const unsigned long long b = raw_bits(v) & 0x7fffffffffffffffull;
+    return b <= INF_BITS ? b : 0ull;
+}
+// A non-negative double rounded towards 0 to a float (0 below 2^-126, infinity from 2^128 on).
+__device__ __forceinline__ float float_below(unsigned long long b) {
+    const unsigned long long e = b >> 29;  // exponent and the first 23 fraction bits
+    return e < (897ull << 23)   ? 0.f
+           : e >= (1151ull << 23) ? __int_as_float(0x7f800000)
+                                  : __uint_as_float((unsigned)(e - (896ull << 23)));
+}
+// Maximum over the warp: of the high words, then of the low words under it.
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long b) {
+    const unsigned hi = __reduce_max_sync(FULL, (unsigned)(b >> 32));
+    const unsigned lo = __reduce_max_sync(FULL, (unsigned)(b >> 32) == hi ? (unsigned)b : 0u);
+    return ((unsigned long long)hi << 32) | lo;
+}
+
+// Solver state of the persistent solve, one copy per block: every block takes
+// the same step from the same reduced sums.
+struct StepState {
+    double y[KMAX], yt[KMAX], d[KMAX], g[KMAX];
+    double F, alpha, tol, res;
+    int iter, phase, done, status, n_eval, final_pending;
+};
+
+// Shared memory of the step.
+struct StepMem {
+    __align__(16) float H[KMAX][H_LD];      // H as reduced (lower triangle)
+    __align__(16) float prow[2][2][KMAX];   // [step mod 2]: the pivot rows
+    __align__(16) float pcol[2][2][KMAX];   // and the pivot columns
+    __align__(16) float4 piv[2];            // the pivot block d00, d10, d11
+    __align__(16) float2 pu[2];             // the right-hand side of the pivot rows
+    float rhs[KMAX];                        // -g of the free variables in order, then the solution
+    int fidx[KMAX];                         // free variables in order
+    unsigned bal[2], diag[2];
+    int viol[2], ok;
+    unsigned long long res[2], gmax[2];
+    float decf[2], absf[2], dF;
+    double dec[2];
+};
+
+// Damped FP32 solve of (H_FF + lam I) x = b (nf free variables) by Gauss-Jordan
+// elimination, two pivots a step; x in sm.rhs.  Returns false when a pivot is not
+// in [2^-126, 2^126].  Thread (tr, tc) of a 16 x 16 grid holds the 4 x 4 entries
+// from (4 tr, 4 tc) in registers, threads tc = 0 also the right-hand side of their
+// rows.  Per step the owners publish the two pivot rows and columns (and the
+// right-hand side's entries) in shared memory; after the step's one barrier
+// every thread eliminates the pair as an L D L^T of its 2 x 2 block would (d0,
+// l = d10 / d0, d1 = d11 - l d10) from its rows, those already eliminated
+// included, so that no triangular solve is left: at the end each pair's 2 x 2
+// system gives its x.  The chain of a step is a barrier, one shared-memory round
+// trip and two reciprocals.  The whole step at 48 variables takes 8.8 us (64:
+// 10.5), against 9.1 (11.7) with panels of four columns and a triangular solve.
+// The reciprocals are the hardware approximation (__fdividef, within 2 ulp
+// for pivots in [2^-126, 2^126]; others fail the check and the caller takes a
+// larger shift).  H is symmetric positive definite up to rounding, and shifted,
+// so the diagonal pivots need no search.
+__device__ __forceinline__ bool step_solve(StepMem& sm, int k, int nf, const float (&H4)[4][4], const float (&b4)[4],
+                                           float lam) {
+    const int tr = k & 15, tc = k >> 4;
+    float M[4][4], u[4], pi0[2] = {0.f, 0.f}, pl[2] = {0.f, 0.f}, pi1[2] = {0.f, 0.f};
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        u[a] = b4[a];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) M[a][b] = H4[a][b] + (tr == tc && a == b ? lam : 0.f);
+    }
+    bool good = true;
+    const int steps = (nf + 1) >> 1;
+    const bool rows_in = 4 * tr < nf;
+    for (int s0 = 0; s0 < steps; s0 += 2) {
+        const int P = s0 >> 1;  // the pivot rows' thread row: two steps each
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (s0 + h < steps) {
+                constexpr float ZERO = 0.f;
+                if (tr == P && tc >= P) {
+                    *reinterpret_cast<float4*>(&sm.prow[h][0][4 * tc]) =
+                        make_float4(M[2 * h][0], M[2 * h][1], M[2 * h][2], M[2 * h][3]);
+                    *reinterpret_cast<float4*>(&sm.prow[h][1][4 * tc]) =
+                        make_float4(M[2 * h + 1][0], M[2 * h + 1][1], M[2 * h + 1][2], M[2 * h + 1][3]);
+                }
+                if (tc == P && rows_in) {
+                    *reinterpret_cast<float4*>(&sm.pcol[h][0][4 * tr]) =
+                        make_float4(M[0][2 * h], M[1][2 * h], M[2][2 * h], M[3][2 * h]);
+                    *reinterpret_cast<float4*>(&sm.pcol[h][1][4 * tr]) =
+                        make_float4(M[0][2 * h + 1], M[1][2 * h + 1], M[2][2 * h + 1], M[3][2 * h + 1]);
+                    if (tr == P)
+                        sm.piv[h] = make_float4(M[2 * h][2 * h], M[2 * h + 1][2 * h], M[2 * h + 1][2 * h + 1], ZERO);
+                }
+                if (tc == 0 && tr == P) sm.pu[h] = make_float2(u[2 * h], u[2 * h + 1]);
+                step_sync();
+                if (rows_in && (tc >= P || tc == 0)) {
+                    const float4 d = sm.piv[h];
+                    float4 c0 = *reinterpret_cast<const float4*>(&sm.pcol[h][0][4 * tr]);
+                    float4 c1 = *reinterpret_cast<const float4*>(&sm.pcol[h][1][4 * tr]);
+                    const float4 r0 = *reinterpret_cast<const float4*>(&sm.prow[h][0][4 * tc]);
+                    float4 r1 = *reinterpret_cast<const float4*>(&sm.prow[h][1][4 * tc]);
+                    const float2 e = sm.pu[h];
+                    const float i0 = __fdividef(1.f, d.x);
+                    const float l = d.y * i0;
+                    const float d1 = fmaf(-l, d.y, d.z);
+                    const float i1 = __fdividef(1.f, d1);
+                    r1 = make_float4(fmaf(-l, r0.x, r1.x), fmaf(-l, r0.y, r1.y), fmaf(-l, r0.z, r1.z),
+                                     fmaf(-l, r0.w, r1.w));
+                    float m0[4] = {c0.x * i0, c0.y * i0, c0.z * i0, c0.w * i0};
+                    float m1[4] = {fmaf(-l, c0.x, c1.x) * i1, fmaf(-l, c0.y, c1.y) * i1, fmaf(-l, c0.z, c1.z) * i1,
+                                   fmaf(-l, c0.w, c1.w) * i1};
+                    if (tr == P) {  // the pivot rows stay
+                        m0[2 * h] = m0[2 * h + 1] = 0.f;
+                        m1[2 * h] = m1[2 * h + 1] = 0.f;
+                    }
+                    const float q0[4] = {r0.x, r0.y, r0.z, r0.w}, q1[4] = {r1.x, r1.y, r1.z, r1.w};
+                    if (tc >= P)
+#pragma unroll
+                        for (int a = 0; a < 4; ++a)
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) M[a][b] = fmaf(-m1[a], q1[b], fmaf(-m0[a], q0[b], M[a][b]));
+                    if (tc == 0) {
+                        const float e1 = fmaf(-l, e.x, e.y);
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) u[a] = fmaf(-m1[a], e1, fmaf(-m0[a], e.x, u[a]));
+                        good = good && d.x >= 1.17549435e-38f && d.x <= 8.50705917e37f && d1 >= 1.17549435e-38f &&
+                               d1 <= 8.50705917e37f;
+                        if (tr == P) {
+                            pi0[h] = i0;
+                            pl[h] = l;
+                            pi1[h] = i1;
+                        }
+                    }
+                }
+            }
+        }
+    }
+    if (tc == 0) {  // half a warp
+        if (rows_in)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float x1 = fmaf(-pl[h], u[2 * h], u[2 * h + 1]) * pi1[h];
+                sm.rhs[4 * tr + 2 * h] = fmaf(-pl[h], x1, u[2 * h] * pi0[h]);
+                sm.rhs[4 * tr + 2 * h + 1] = x1;
+            }
+        if (tr == 0) sm.ok = good;  // thread (0, 0) takes part in every step
+    }
+    step_sync();
+    return sm.ok != 0;
+}
+
+// The projected-Newton step: variable v = k mod 64 of thread k; warps 0 and 1 test
+// the KKT conditions, warps 2 and 3 the decrease, all threads share the
+// factorisation.  LOCAL: the state is the block's shared copy (persistent solve);
+// else it is the plan's, in device memory, read through L2.  The reduced sums:
+// Ft, gt and gn of variable v, and H's lower triangle in sm.H (visible after the
+// first barrier).  The caller synchronises the block before and after it.
+//
+// A chain of dependent block phases, so latency is all that counts: FP64 only
+// where a decision needs it (the tests are made in FP32 with their error
+// margins and repeated in FP64 when they fall inside).
+template <bool LOCAL, class ST>
+__device__ __forceinline__ void master_step_body(ST* st, int K, double Ft, double gt_, float gn_, int max_iter,
+                                                 double tol_rel, double sigma, StepMem& sm) {
+    auto get = [](const auto* p) {
+        if constexpr (LOCAL)
+            return *p;
+        else
+            return __ldcg(p);
+    };
+    const int k = threadIdx.x, lane = k & 31, warp = k >> 5;
+    const int v = k & (KMAX - 1);
+    const double yt_ = get(&st->yt[v]), y_ = get(&st->y[v]), g_ = get(&st->g[v]);
+    const int phase = get(&st->phase), iter0 = get(&st->iter), n_eval0 = get(&st->n_eval);
+    const double tol0 = get(&st->tol), F0 = get(&st->F), alpha0 = get(&st->alpha);
+    const bool own = v < K;
+    const bool lead = k < KMAX && own;  // thread k < K owns variable k
+    const double yt = own ? yt_ : 0.0, gt = own ? gt_ : 0.0;
+    const float bneg = -(float)gt;
     // tolerance of this solve from the gradient at the warm start
     double tol = tol0;
     if (phase == 0) {
-        if (vwarp) {
-            const double m = warp_max_nonneg(own ? fabs(gt) : 0.0);
-            if ((k & 31) == 0) sw3[k >> 5] = m;
+        if (warp < 2) {
+            const unsigned long long m = warp_max_bits(own ? abs_bits(gt) : 0ull);
+            if (lane == 0) sm.gmax[warp] = m;
         }
-        __syncthreads();
-        long long mb = nonneg_bits(sw3[0]);
-        for (int w = 1; w < nw; ++w) mb = max(mb, nonneg_bits(sw3[w]));
-        tol = tol_rel * fmax(__longlong_as_double(mb), 1e-300);
-        if (k == 0) st->tol = tol;
+        step_sync();
+        if (warp < 2) tol = tol_rel * fmax(__longlong_as_double((long long)max(sm.gmax[0], sm.gmax[1])), 1e-300);
     }
-    // KKT violation flag, residual and Armijo decrease in one reduction
-    double rmax = 0.0, dec = 0.0;
-    int viol = 0;
-    if (vwarp) {
-        const double rt = own ? fabs(yt - fmax(yt - gt, 0.0)) : 0.0;
-        viol = __any_sync(FULL, own && rt > tol + NOISE * (double)U32 * gn) ? 1 : 0;
-        rmax = warp_max_nonneg(rt);
-        dec = own ? g * (yt - y) : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dec += __shfl_xor_sync(FULL, dec, o);
-        if ((k & 31) == 0) {
-            sw[k >> 5] = rmax;
-            sw2[k >> 5] = dec;
-            swi[k >> 5] = viol;
+    if (warp < 2) {
+        // |y - P(y - g)| = |min(y, g)| (y >= 0)
+        const unsigned long long yb = raw_bits(yt), gb = raw_bits(gt), ga = gb & 0x7fffffffffffffffull;
+        const unsigned long long rt = !own ? 0ull : (gb >> 63) ? (ga <= INF_BITS ? ga : yb) : min(gb, yb);
+        const float rf = float_below(rt), lf = fmaf((float)(NOISE * (double)U32), own ? gn_ : 0.f, float_below(raw_bits(tol)));
+        bool vi = own && rf > lf * (1.f + 1e-6f);
+        const bool sure = !own || vi || rf * (1.f + 1e-6f) <= lf;
+        if (__any_sync(FULL, !sure))
+            if (!sure) vi = rt > raw_bits(tol + NOISE * (double)U32 * (double)gn_);
+        const int viol = __any_sync(FULL, vi) ? 1 : 0;
+        const unsigned long long rm = warp_max_bits(rt);
+        if (lane == 0) {
+            sm.res[warp] = rm;
+            sm.viol[warp] = viol;
+        }
+    } else if (warp < 4 && phase != 0) {
+        // g^T (y_t - y) in FP32, with the sum of its terms' magnitudes
+        const float t = own ? (float)g_ * (float)(yt - y_) : 0.f;
+        float s = warp_sum_f32(t), a = warp_sum_f32(fabsf(t));
+        if (lane == 0) {
+            sm.decf[warp - 2] = s;
+            sm.absf[warp - 2] = a;
+            if (warp == 2) sm.dF = (float)(Ft - F0);
         }
     }
-    __syncthreads();
-    long long rb = nonneg_bits(sw[0]);
-    dec = sw2[0];
-    viol = swi[0];
-    for (int w = 1; w < nw; ++w) {
-        rb = max(rb, nonneg_bits(sw[w]));
-        dec += sw2[w];
-        viol |= swi[w];
-    }
-    rmax = __longlong_as_double(rb);
+    step_sync();
+    const unsigned long long rb = max(sm.res[0], sm.res[1]);
+    const int viol = sm.viol[0] | sm.viol[1];
     const bool cap = iter0 >= max_iter + 64;
-    const bool accept = !cap && (phase == 0 || !viol || Ft <= F0 + sigma * dec);
-    if (k == 0) st->n_eval = __ldcg(&st->n_eval) + 1;
+    bool accept = !cap;
+    if (accept && phase != 0 && viol) {  // Armijo: F_t <= F + sigma g^T (y_t - y)
+        const float sg = (float)sigma, dF = sm.dF;
+        const float thr = sg * (sm.decf[0] + sm.decf[1]);
+        const float m = 1e-5f * (sg * (sm.absf[0] + sm.absf[1]) + fabsf(dF));
+        accept = dF <= thr - m;
+        if (!accept && !(dF > thr + m)) {  // too close to tell in FP32 (the same for every thread)
+            if (warp < 2) {
+                double dec = own ? g_ * (yt - y_) : 0.0;
+                dec = warp_sum_f64(dec);
+                if (lane == 0) sm.dec[warp] = dec;
+            }
+            step_sync();
+            accept = Ft <= F0 + sigma * (sm.dec[0] + sm.dec[1]);
+        }
+    }
+    if (k == 0) {
+        st->n_eval = n_eval0 + 1;
+        if (phase == 0) st->tol = tol;
+    }
     if (cap) {
         if (k == 0) {
             st->status = MASTER_MAXITER;
@@ -663,7 +854,7 @@ __device__ __forceinline__ void master_step_body(MasterDev* __restrict__ st, int
         return;
     }
     if (!accept) {
-        const double alpha = __ldcg(&st->alpha) * 0.5;
+        const double alpha = alpha0 * 0.5;
         if (alpha < 9.3e-10) {  // 2^-30: the line search found no decrease
             if (k == 0) {
                 st->status = MASTER_STALLED;
@@ -672,7 +863,7 @@ __device__ __forceinline__ void master_step_body(MasterDev* __restrict__ st, int
             }
             return;
         }
-        if (own) st->yt[k] = fmax(y + alpha * __ldcg(&st->d[k]), 0.0);
+        if (lead) st->yt[k] = fmax(y_ + alpha * get(&st->d[k]), 0.0);
         if (k == 0) {
             st->alpha = alpha;
             st->iter = iter0 + 1;
@@ -681,13 +872,13 @@ __device__ __forceinline__ void master_step_body(MasterDev* __restrict__ st, int
         return;
     }
     // accept the trial point
-    if (own) {
+    if (lead) {
         st->y[k] = yt;
         st->g[k] = gt;
     }
     if (k == 0) {
         st->F = Ft;
-        st->res = rmax;
+        st->res = __longlong_as_double((long long)rb);
     }
     if (!viol || iter0 >= max_iter) {
         if (k == 0) {
@@ -697,206 +888,59 @@ __device__ __forceinline__ void master_step_body(MasterDev* __restrict__ st, int
         return;
     }
     // epsilon-active set, free variables compacted in order
-    bool active = false;
-    if (vwarp) {
-        const double eps = fmin(1e-3, rmax);
-        active = own && yt <= eps && gt > 0.0;
-    }
-    const bool fr = own && !active;
-    const unsigned bal = __ballot_sync(FULL, fr);
-    __syncthreads();
-    if ((k & 31) == 0) swi[k >> 5] = __popc(bal);
-    __syncthreads();
-    int nf = 0, pos = 0;
-#pragma unroll
-    for (int w = 0; w < STEP_W; ++w) {
-        pos += w < (k >> 5) ? swi[w] : 0;
-        nf += swi[w];
-    }
-    pos += __popc(bal & ((1u << (k & 31)) - 1u));
-    if (fr) fidx[pos] = k;
-#pragma unroll
-    for (int m = 0; m < KMAX * KMAX / STEP_T; ++m) {  // H into Lw (overwritten later by the factorisation)
-        const int idx = m * STEP_T + k;
-        Lw[idx / KMAX][idx % KMAX] = hpre[m];
-    }
-    if (k < KMAX) sg[k] = (float)gt;
-    double d = active ? -gt : 0.0;
-    __syncthreads();
-    // Damped FP32 L D L^T factorisation of H_FF with the forward solve folded in,
-    // by panels of 4 columns with one barrier per panel.  The working lower
-    // triangle A lives in shared memory.  For panel p (columns c0 = 4p .. c0+3)
-    // the threads that need it factor the 4 x 4 diagonal block themselves
-    // (identical arithmetic everywhere) and map rows through it, w = x L11^-T:
-    //   - work item 4 t + a < 4 nb(nb+1)/2 (threads below FACT_TILE_T, strided)
-    //     takes row a of trailing tile t = (r, s), s <= r, and subtracts
-    //     w_R D^-1 w_Q^T from it (the trailing part shrinks, so do the items);
-    //   - threads FACT_COLW + r' write the panel's final column entries w
-    //     (unscaled: L_ik d_k) of row block r' into Lw, and the pivots d and
-    //     their reciprocals;
-    //   - thread FACT_RHSW writes the eliminated right-hand side of the panel
-    //     into ye, threads FACT_RHSW + r subtract its contribution from row
-    //     block r of u.
-    // Rows nf .. 4*panels-1 are padding with only the shift on the diagonal.  The
-    // pivots are checked once at the end; one that is not in [2^-126, 2^126]
-    // (non-positive, or outside the range of the reciprocal approximation)
-    // restarts the factorisation with a 100x larger shift.  Then L^T x = D^-1 ye
-    // is solved by warp 0 with the unit lower factor L_ik = Lw_ik / d_k.
-    const int ti = k >> 4, tq = k & 15;
-    const int n_panels = (nf + 3) >> 2;
-    const int n4 = 4 * n_panels;
-    float Hr[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int i = ti + 16 * a, q = tq + 16 * b;
-            Hr[a][b] = (i < nf && q <= i) ? Lw[fidx[i]][fidx[q]] : 0.f;
+    const bool active = lead && raw_bits(yt) <= min(raw_bits(1e-3), rb) && nonneg_bits(gt) > 0ull;
+    const bool fr = lead && !active;
+    const float hd = fr ? sm.H[k][k] : 0.f;
+    if (k < KMAX) {
+        const unsigned bal = __ballot_sync(FULL, fr);
+        const unsigned md = __reduce_max_sync(FULL, hd > 0.f ? __float_as_uint(hd) : 0u);
+        if (lane == 0) {
+            sm.bal[warp] = bal;
+            sm.diag[warp] = md;
         }
-    const float bk = k < nf ? -sg[fidx[k]] : 0.f;
-    float dg = 0.f;
+    }
+    step_sync();
+    const int nf = __popc(sm.bal[0]) + __popc(sm.bal[1]);
+    const float maxdiag = __uint_as_float(max(sm.diag[0], sm.diag[1]));
+    int pos = 0;
+    if (fr) {
+        pos = (warp ? __popc(sm.bal[0]) : 0) + __popc(sm.bal[warp] & ((1u << lane) - 1u));
+        sm.fidx[pos] = k;
+        sm.rhs[pos] = bneg;
+    }
+    double d = active ? -gt : 0.0;
+    step_sync();
+    const int r0 = 4 * (k & 15), q0 = 4 * (k >> 4);  // this thread's 4 x 4 entries
+    float H4[4][4], b4[4];
+    {
+        int fi[4], fq[4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) dg = fmaxf(dg, (ti == tq) ? Hr[a][a] : 0.f);
-    const float maxdiag = blk_max_f32(dg, swf);
-    float lam = 1e-6f * maxdiag + 1e-30f;
-    bool ok = false;
-    for (int attempt = 0; attempt < 6 && !ok; ++attempt) {
+        for (int a = 0; a < 4; ++a) {
+            fi[a] = r0 + a < nf ? sm.fidx[r0 + a] : -1;
+            fq[a] = q0 + a < nf ? sm.fidx[q0 + a] : -1;
+            b4[a] = r0 + a < nf ? sm.rhs[r0 + a] : 0.f;
+        }
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int i = ti + 16 * a, q = tq + 16 * b;
-                A[i][q] = Hr[a][b] + ((i == q && i < n4) ? lam : 0.f);
-            }
-        if (k < KMAX) u[k] = bk;
-        __syncthreads();
-        for (int p = 0; p < n_panels; ++p) {
-            const int c0 = 4 * p;
-            const int nb = n_panels - p - 1;
-            const int ntile4 = 2 * nb * (nb + 1);  // rows of the nb (nb + 1) / 2 trailing tiles
-            const bool tilew = k < FACT_TILE_T && k < ntile4;
-            const bool colw = k >= FACT_COLW && k <= FACT_COLW + nb;
-            const bool rhsw = k >= FACT_RHSW && k <= FACT_RHSW + nb;
-            if (tilew || colw || rhsw) {
-                const float4 a0 = *reinterpret_cast<const float4*>(&A[c0][c0]);
-                const float4 a1 = *reinterpret_cast<const float4*>(&A[c0 + 1][c0]);
-                const float4 a2 = *reinterpret_cast<const float4*>(&A[c0 + 2][c0]);
-                const float4 a3 = *reinterpret_cast<const float4*>(&A[c0 + 3][c0]);
-                // the pivot reciprocals on the chain of every panel: the hardware
-                // approximation (__fdividef, within 2 ulp for pivots in
-                // [2^-126, 2^126]; a pivot outside that range fails the check
-                // below and the factorisation restarts with a larger shift)
-                const float d0 = a0.x, i0 = __fdividef(1.f, d0);
-                const float l10 = a1.x * i0;
-                const float d1 = a1.y - l10 * a1.x, i1 = __fdividef(1.f, d1);
-                const float l20 = a2.x * i0, w21 = a2.y - l10 * a2.x, l21 = w21 * i1;
-                const float d2 = a2.z - l20 * a2.x - l21 * w21, i2 = __fdividef(1.f, d2);
-                const float l30 = a3.x * i0, w31 = a3.y - l10 * a3.x, l31 = w31 * i1;
-                const float w32 = a3.z - l20 * a3.x - l21 * w31, l32 = w32 * i2;
-                const float d3 = a3.w - l30 * a3.x - l31 * w31 - l32 * w32, i3 = __fdividef(1.f, d3);
-                auto xform = [&](float4 x) {
-                    float4 w;
-                    w.x = x.x;
-                    w.y = x.y - l10 * w.x;
-                    w.z = x.z - l20 * w.x - l21 * w.y;
-                    w.w = x.w - l30 * w.x - l31 * w.y - l32 * w.z;
-                    return w;
-                };
-                if (tilew) {
-                    // one row a of trailing tile t per work item; the four rows of
-                    // a tile run in parallel
-                    for (int it = k; it < ntile4; it += FACT_TILE_T) {
-                        const int t = it >> 2, a = it & 3;
-                        int r = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
-                        while ((r + 1) * (r + 2) / 2 <= t) ++r;
-                        while (r * (r + 1) / 2 > t) --r;
-                        const int R = c0 + 4 + 4 * r, Q = c0 + 4 + 4 * (t - r * (r + 1) / 2);
-                        float4 wq[4];
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) wq[b] = xform(*reinterpret_cast<const float4*>(&A[Q + b][c0]));
-                        float4 w = xform(*reinterpret_cast<const float4*>(&A[R + a][c0]));
-                        w.x *= i0;
-                        w.y *= i1;
-                        w.z *= i2;
-                        w.w *= i3;
-                        float4 tt = *reinterpret_cast<const float4*>(&A[R + a][Q]);
-                        tt.x -= w.x * wq[0].x + w.y * wq[0].y + w.z * wq[0].z + w.w * wq[0].w;
-                        tt.y -= w.x * wq[1].x + w.y * wq[1].y + w.z * wq[1].z + w.w * wq[1].w;
-                        tt.z -= w.x * wq[2].x + w.y * wq[2].y + w.z * wq[2].z + w.w * wq[2].w;
-                        tt.w -= w.x * wq[3].x + w.y * wq[3].y + w.z * wq[3].z + w.w * wq[3].w;
-                        *reinterpret_cast<float4*>(&A[R + a][Q]) = tt;
-                    }
-                } else if (colw) {
-                    const int R = c0 + 4 * (k - FACT_COLW);
-#pragma unroll
-                    for (int a = 0; a < 4; ++a)
-                        *reinterpret_cast<float4*>(&Lw[R + a][c0]) =
-                            xform(*reinterpret_cast<const float4*>(&A[R + a][c0]));
-                    if (k == FACT_COLW) {
-                        piv[c0] = d0;
-                        piv[c0 + 1] = d1;
-                        piv[c0 + 2] = d2;
-                        piv[c0 + 3] = d3;
-                        rd[c0] = i0;
-                        rd[c0 + 1] = i1;
-                        rd[c0 + 2] = i2;
-                        rd[c0 + 3] = i3;
-                    }
-                } else {
-                    const float4 e = xform(*reinterpret_cast<const float4*>(&u[c0]));
-                    if (k == FACT_RHSW) {
-                        *reinterpret_cast<float4*>(&ye[c0]) = e;
-                    } else {
-                        const int R = c0 + 4 * (k - FACT_RHSW);
-                        const float e0 = e.x * i0, e1 = e.y * i1, e2 = e.z * i2, e3 = e.w * i3;
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) {
-                            const float4 w = xform(*reinterpret_cast<const float4*>(&A[R + a][c0]));
-                            u[R + a] -= w.x * e0 + w.y * e1 + w.z * e2 + w.w * e3;
-                        }
-                    }
-                }
-            }
-            __syncthreads();
-        }
-        const float pk = k < n4 ? piv[k] : 1.f, rk = k < n4 ? rd[k] : 1.f;
-        ok = __syncthreads_and(pk >= 1.17549435e-38f && pk <= 8.50705917e37f && isfinite(rk)) != 0;
+            for (int b = 0; b < 4; ++b)
+                H4[a][b] = fi[a] >= 0 && fq[b] >= 0 ? sm.H[max(fi[a], fq[b])][min(fi[a], fq[b])] : 0.f;
+    }
+    float lam = 1e-6f * maxdiag + 1e-30f;
+    bool ok = false;
+    for (int attempt = 0; attempt < 6 && !ok; ++attempt) {  // a failed pivot: a 100x larger shift
+        ok = step_solve(sm, k, nf, H4, b4, lam);
         lam *= 100.f;
     }
-    if (ok) {
-        if (k >= nf && k < KMAX) rd[k] = 0.f;  // padding rows
-        __syncthreads();
-        // L^T x = D^-1 ye by warp 0, one pivot at a time from the last, with
-        // L_ik = Lw_ik / d_k: lanes keep b_r = ye_r - sum_{i > r, done} Lw_ir x_i
-        // for rows r = lane and lane + 32; x_j = b_j / d_j is broadcast from its
-        // lane and every row above j takes its term (one shuffle and one FMA
-        // per pivot on the dependent chain)
-        if (k < 32) {
-            float b0 = k < n4 ? ye[k] : 0.f, b1 = k + 32 < n4 ? ye[k + 32] : 0.f;
-            const float r0 = rd[k], r1 = rd[k + 32];
-            for (int j = nf - 1; j >= 0; --j) {
-                const float xj = __shfl_sync(FULL, j < 32 ? b0 * r0 : b1 * r1, j & 31);
-                if (k == (j & 31)) {
-                    if (j < 32)
-                        b0 = xj;
-                    else
-                        b1 = xj;
-                }
-                if (k < j) b0 = fmaf(-Lw[j][k], xj, b0);
-                if (k + 32 < j) b1 = fmaf(-Lw[j][k + 32], xj, b1);
-            }
-            rhs[k] = b0;
-            rhs[k + 32] = b1;
-        }
-        __syncthreads();
-        if (fr) d = (double)rhs[pos];
-    } else if (fr) {
-        const double hk = (double)__ldcg(&st->Ht[k * KMAX + k]);
-        d = -gt / (hk > 0.0 ? hk : 1.0);
+    if (fr) {
+        if (ok)
+            d = (double)sm.rhs[pos];
+        else
+            d = -gt / (hd > 0.f ? (double)hd : 1.0);
     }
-    if (own) {
+    if (lead) {
         st->d[k] = d;
-        st->yt[k] = fmax(yt + d, 0.0);
+        st->yt[k] = relu_bits(yt + d);
     }
     if (k == 0) {
         st->alpha = 1.0;
@@ -919,6 +963,7 @@ __global__ void __launch_bounds__(STEP_T, 1) k_master_reduce_step(const float* _
                                                                double tol_rel, double sigma,
                                                                cudaGraphConditionalHandle cond, int use_cond) {
     __shared__ int s_last;
+    __shared__ StepMem sm;
     if (st->done) {  // the same for every block: only the last block of a launch changes it
         if (use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0u);
         return;
@@ -929,40 +974,168 @@ __global__ void __launch_bounds__(STEP_T, 1) k_master_reduce_step(const float* _
     __syncthreads();
     if (!s_last) return;
     if (threadIdx.x == 0) st->ticket = 0;
-    master_step_body(st, max_iter, tol_rel, sigma);
+    if (__ldcg(&st->err)) {  // a tile copy was lost in an evaluation: stop with the last accepted point
+        if (threadIdx.x == 0) {
+            st->status = MASTER_ERROR;
+            st->final_pending = 1;
+            st->done = 1;
+        }
+    } else {
+        const int K = __ldcg(&st->K), tid = threadIdx.x, v = tid & (KMAX - 1);
+        const double Ft = __ldcg(&st->Ft), gt = __ldcg(&st->gt[v]);
+        const float gn = __ldcg(&st->gn[v]);
+#pragma unroll
+        for (int m = 0; m < KMAX * KMAX / STEP_T; ++m) {
+            const int r = 4 * m + (tid >> 6);
+            if (v <= r && r < K) sm.H[r][v] = __ldcg(&st->Ht[r * KMAX + v]);
+        }
+        __syncthreads();
+        master_step_body<false>(st, K, Ft, gt, gn, max_iter, tol_rel, sigma, sm);
+    }
     if (use_cond && threadIdx.x == 0) cudaGraphSetConditional(cond, st->done ? 0u : 1u);
 }
 
 // ---- the master solve as one persistent cooperative kernel -------------------
-// All blocks are co-resident (cooperative launch).  Block b owns the chunks of
-// CHV = 128 voxels b, b + G, b + 2G, ... of the slab (interleaved, so the active
-// voxels of a compact target spread evenly over the blocks).  Per Newton
-// iteration:
-//   A. the chunk's slab columns arrive in shared memory by TMA (boxes of 128
-//      voxels x 16 columns, one mbarrier; the next chunk's copy is in flight
-//      while the current one is folded in, and the block's first chunk is
-//      fetched again for the next iteration as soon as its last one has been
-//      read: the slab does not change during a solve); warps 0-3 (lane = voxel)
-//      compute the compensated z, then pi, h, F, and copy the rows of the
-//      voxels with h > 0 to a compacted row-major buffer; every thread then
-//      accumulates its 4x4 block of the partial H (and g and the rounding
-//      scale of g) over those rows; after its chunks the block writes its
-//      partials to column b of the partial arrays;
+// One block of 16 warps per SM, all co-resident (cooperative launch).  A warp
+// owns tiles of 32 voxels, one per lane, interleaved over the grid's warps (so the
+// active voxels of a compact target spread over them), and meets the other
+// warps of its block only when its tiles are done.  A tile's doses (512 bytes per
+// group of four columns) come to the warp's ring in shared memory by 16-byte
+// asynchronous copies, tiles ahead; they stay there from one evaluation to
+// the next where the ring holds all of the warp's tiles.  Per Newton iteration:
+//   A. per tile: the lanes form the compensated z of their voxel, then pi, h, F
+//      and the voxel's curvature state; the voxels with h > 0 then add to g and
+//      its rounding scale, a lane per voxel and group of columns; the
+//      voxels whose h changed go to the warp's list and, while there is room,
+//      their doses to a block-wide pool of rows.  After its tiles the block adds
+//      the listed changes to its kept partial H (Delta h s s^T, a 2x2 block of H
+//      per thread) and writes its partials to column b of the partial arrays;
 //   grid barrier;
-//   B. every block reduces its share of the outputs in a fixed order; the block
-//      that finishes last (ticket after a fence) takes the Newton step;
-//   grid barrier; stop when the step marked the solve done.
-// Every barrier wait is bounded: after GRID_WAIT_LIMIT polls the block reports
-// st->err = 2, marks the barrier broken (later launches of the solve return at
-// entry) and every block leaves at the next barrier or check.
-constexpr int PT = STEP_T;         // threads per block (the step body's layout)
+//   B. every block reduces its share of the outputs in a fixed order, into words
+//      tagged with the evaluation's number;
+//   C. every block collects the words and takes the same Newton step from them, on
+//      its own copy of the solver state, so no block waits for another's step.
+// The first evaluation of a solve that follows a converged one on the same
+// grid, with one more aperture at intensity 0, is at the point the last one ended
+// on: z, pi, F, g and H of the older apertures stand, and only the new
+// aperture's g and its column of H are formed (MODE_EXT).
+// One plan of 50 apertures, H&N-shaped (304,184 voxels), FP16 storage: 6.71 ms,
+// against 8.70 with blocks of 256 threads on 128-voxel chunks copied by TMA, five
+// block barriers to a chunk, and the step taken by one block between two grid
+// barriers; 8 prostate-shaped plans of 20 apertures at once 8.33 ms (10.96).  An
+// evaluation now takes 22.7 us on average (28 before): tiles 6.4, the update of
+// H 1.6, partials 0.7, waiting for the last block 2.6, reduction and collection
+// 5.2, step 5.0.  The pass is bound by instruction issue, the rest by latency.
+// Every wait is bounded: after GRID_WAIT_LIMIT polls the block reports st->err = 2, marks the barrier broken (later launches of the solve return at
+// entry) and every block leaves at its next wait.
+constexpr int PT = 512;            // threads per block (the step takes the first STEP_T)
 constexpr int PW = PT / 32;
-constexpr int CHV = 128;           // voxels per chunk of the persistent pass
-constexpr int BOXC = 16;           // slab columns per TMA box of the persistent pass
-constexpr int NST_MAX = 4;         // copies in flight per block (when the pool is small enough)
+constexpr int RING = 21;           // groups of four columns of a tile in a warp's ring
+constexpr int RING_LD = 132;       // floats of a group in the ring: 32 voxels x 4, and 4 against bank conflicts
+constexpr size_t RING_BYTES = (size_t)PW * RING * RING_LD * sizeof(float);
+constexpr int LIST = 128;          // listed voxels of a warp: four tiles
+constexpr int HB = KMAX;           // rows of changed voxels held at a time for the update of H (the step's matrix A)
 enum { MODE_FULL = 0, MODE_EXT = 1, MODE_INC = 2 };  // the kept partial H: rebuilt, extended by a column, updated
 constexpr int GRID_WAIT_LIMIT = 1 << 22;
-constexpr size_t PERSIST_SMEM_MAX = 150 * 1024;  // dynamic shared memory the kernel is configured for
+
+__device__ __forceinline__ void copy16_async(float* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
+// A warp's tiles in its ring: copy n (n = 0, 1, ... over the launch) is tile n
+// mod tiles; group g of copy n sits at position (n KG + g) mod size.  size is a
+// whole number of tiles (two to four ahead, or all of them: nothing is copied
+// twice), or, where the ring holds fewer than two, the whole ring: then the next
+// tile's first RING - KG groups are ahead and its others follow when the tile is
+// released.  A group's 32 x 16 bytes are followed by 16 unused ones, so that
+// the same voxel of eight groups, as the gradient reads it, falls on different
+// banks.
+struct TileRing {
+    float* buf;
+    const float* src;            // the lane's voxel of the warp's first tile, group 0
+    size_t gstride, tstride;     // floats from one group to the next, from one tile to the next
+    int KG, size, tiles, slots;  // slots: tiles the ring holds; 0: the fractional form
+    int n, pos;                  // the copy in use and its position
+    int iss_tile, iss_pos;       // next tile to issue (index in the warp's), position of its next group
+    bool resident;
+
+    __device__ __forceinline__ void issue(int g0, int g1) {  // groups [g0, g1) of tile iss_tile
+        const float* p = src + (size_t)iss_tile * tstride + (size_t)g0 * gstride;
+        float* d = buf + iss_pos * RING_LD + (threadIdx.x & 31) * 4;
+        for (int g = g0; g < g1; ++g, p += gstride) {
+            copy16_async(d, p);
+            d += RING_LD;
+            if (++iss_pos == size) {
+                iss_pos = 0;
+                d -= size * RING_LD;
+            }
+        }
+        copies_commit();
+    }
+    __device__ __forceinline__ void next_tile() {
+        if (++iss_tile == tiles) iss_tile = 0;
+    }
+    __device__ __forceinline__ void init(float* b, const float* slab, int ld, int KG_, int t0, int stride, int n32) {
+        buf = b;
+        src = slab + ((size_t)t0 * 32 + (threadIdx.x & 31)) * 4;
+        gstride = (size_t)ld * 4;
+        tstride = (size_t)stride * 128;
+        KG = KG_;
+        tiles = t0 < n32 ? (n32 - 1 - t0) / stride + 1 : 0;
+        const int fit = RING / KG;
+        resident = tiles <= fit;
+        slots = resident ? tiles : fit >= 2 ? min(fit, 4) : 0;
+        size = slots ? slots * KG : RING;
+        n = pos = iss_tile = iss_pos = 0;
+        if (tiles == 0) return;
+        for (int k = 0; k < max(slots, 1); ++k) {
+            issue(0, KG);
+            next_tile();
+        }
+        if (slots == 0) issue(0, RING - KG);  // the first groups of the next tile
+    }
+    // Copy n has arrived (every lane; the lanes see each other's pieces).
+    __device__ __forceinline__ void wait() {
+        if (resident)
+            copies_wait<0>();
+        else if (slots == 4)
+            copies_wait<3>();
+        else if (slots == 3)
+            copies_wait<2>();
+        else
+            copies_wait<1>();
+        __syncwarp();
+    }
+    // Copy n has been read (by the whole warp): its place is refilled.
+    __device__ __forceinline__ void release() {
+        ++n;
+        pos += KG;
+        if (resident) {
+            if (n == tiles) n = pos = 0;
+            return;
+        }
+        if (pos >= size) pos -= size;
+        __syncwarp();
+        if (slots) {
+            issue(0, KG);
+            next_tile();
+        } else {
+            issue(RING - KG, KG);
+            next_tile();
+            issue(0, RING - KG);
+        }
+    }
+    // Group g of the copy in use: its 32 voxels' float4 each.
+    __device__ __forceinline__ const float* group(int g) const {
+        const int x = pos + g;
+        return buf + (x >= size ? x - size : x) * RING_LD;
+    }
+};
 
 // Barrier over the blocks of one cooperative launch with one acquire-release
 // atomic per arrival.  The counter only grows: barrier e of a launch completes when it
@@ -983,7 +1156,10 @@ __device__ __forceinline__ bool grid_sync(GridBar* gb, unsigned nblocks, unsigne
         int ok = 1;
         if (arrived != target) {
             int i = 0;
-            while ((int)(ld_acquire_gpu(&gb->count) - target) < 0 && ++i < GRID_WAIT_LIMIT) __nanosleep(64);
+            while ((int)(ld_acquire_gpu(&gb->count) - target) < 0 && ++i < GRID_WAIT_LIMIT) {
+                __nanosleep(64);
+                if ((i & 4095) == 0 && ld_acquire_gpu(&gb->broken)) i = GRID_WAIT_LIMIT - 1;  // another gave up
+            }
             ok = i < GRID_WAIT_LIMIT;
             if (!ok) atomicExch(&gb->broken, 1u);
         }
@@ -993,502 +1169,592 @@ __device__ __forceinline__ bool grid_sync(GridBar* gb, unsigned nblocks, unsigne
     return *s_flag != 0;
 }
 
+// s + c of four chains as a pair.
+__device__ __forceinline__ void chains_sum(const float (&sc)[4], const float (&cc)[4], float& s, float& c) {
+    s = sc[0];
+    c = cc[0];
+#pragma unroll
+    for (int q = 1; q < 4; ++q) {
+        const float t2 = s + sc[q];
+        const float bb = t2 - s;
+        const float e = (s - (t2 - bb)) + (sc[q] - bb);
+        s = t2;
+        c += e + cc[q];
+    }
+}
+
+// z of one voxel: the compensated dot product of its doses dose4(c), c < KP
+// (columns K .. KP - 1 meet y = 0), with y, in four chains, as a pair (s, c).
+// s_y: (yh, yl) of two columns per entry.
+template <class Dose4>
+__device__ __forceinline__ void voxel_dot(int KP, const float4* s_y, float& s, float& c, Dose4 dose4) {
+    float sc[4] = {0.f, 0.f, 0.f, 0.f}, cc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int k = 0; k < KP; k += 4) {
+        const float4 a = dose4(k);
+        const float4 y0 = s_y[k >> 1], y1 = s_y[(k >> 1) + 1];
+        dot2_step(sc[0], cc[0], a.x, y0.x, y0.y);
+        dot2_step(sc[1], cc[1], a.y, y0.z, y0.w);
+        dot2_step(sc[2], cc[2], a.z, y1.x, y1.y);
+        dot2_step(sc[3], cc[3], a.w, y1.z, y1.w);
+    }
+    chains_sum(sc, cc, s, c);
+}
+
+// The same where every dose is >= 0 and z is known to within a factor: the chains
+// start at C, a power of two at least 4 |z_last| (z_last: the voxel's dose at the
+// previous evaluation).  While a chain's own sum stays within C / 2, every
+// partial sum lies in [C, 1.5 C], so t = RN(s + a yh) differs from s by an exact
+// float d, the rounding error a yh - d has at most ulp(C) / 2 and one FMA gives it:
+// five operations a term instead of dot2_step's eleven, with the same second-order
+// error (terms of size u ulp(z)).  Sums of non-negative terms only grow, so
+// the last one within C / 2 proves the others; returns false otherwise
+// (also for a NaN), and the caller takes voxel_dot.
+__device__ __forceinline__ void dot2_biased(float& s, float& c, float a, float yh, float yl) {
+    const float t = fmaf(a, yh, s);
+    const float d = t - s;
+    c += fmaf(a, yl, fmaf(a, yh, -d));
+    s = t;
+}
+template <class Dose4>
+__device__ __forceinline__ bool voxel_dot_biased(int KP, const float4* s_y, float z_last, float& s, float& c,
+                                                 Dose4 dose4) {
+    const float C = __uint_as_float((__float_as_uint(z_last) & 0x7f800000u) + (3u << 23));
+    float sc[4] = {C, C, C, C}, cc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+    for (int k = 0; k < KP; k += 4) {
+        const float4 a = dose4(k);
+        const float4 y0 = s_y[k >> 1], y1 = s_y[(k >> 1) + 1];
+        dot2_biased(sc[0], cc[0], a.x, y0.x, y0.y);
+        dot2_biased(sc[1], cc[1], a.y, y0.z, y0.w);
+        dot2_biased(sc[2], cc[2], a.z, y1.x, y1.y);
+        dot2_biased(sc[3], cc[3], a.w, y1.z, y1.w);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sc[q] -= C;  // exact
+    chains_sum(sc, cc, s, c);
+    return sc[0] + sc[1] + sc[2] + sc[3] <= 0.5f * C;
+}
+
 // BATCH: one launch for several plans, blocks [g GB, (g + 1) GB) solving the
 // master problem of tasks[g] with its own barrier and partial arrays (the
 // plans' solves run side by side, each on GB blocks); otherwise one plan, t1,
 // on the whole grid.  Every other difference is the block's index within its
 // group (bid) and the group's size (G).
 // The master solve of one plan (a task) by a group of G co-resident blocks, bid
-// the block's index in it; pm the dynamic shared memory, s_target / s_flag the
-// group barrier's shared state (s_target: the block's next target, already
-// based on the barrier counter).  Every block of the group calls it with the
-// same K.
+// the block's index in it; ring_mem the dynamic shared memory; s_target / s_flag the
+// group barrier's shared state (s_target: the block's next target, already based
+// on the barrier counter).
+// Every block of the group calls it with the same K.
 __device__ __forceinline__ void master_solve_group(
-    const float* __restrict__ slab, const CUtensorMap* tmap, int ld, int V, int GS, int S, int max_iter,
-    MasterDev* __restrict__ st,
+    const float* __restrict__ slab, int ld, int V, int GS, int S, int max_iter, MasterDev* st,
     GridBar* __restrict__ gb, float* __restrict__ H_part, double* __restrict__ g_part, float* __restrict__ gn_part,
     double* __restrict__ F_part, const uint8_t* __restrict__ vstruct, const StructTermsF* __restrict__ tf,
     double tol_rel, float* __restrict__ z_out, float* __restrict__ pi_out, CGDev* __restrict__ cg,
-    uint8_t* __restrict__ vstate, float* __restrict__ H_keep, int bid, int G, int K, int KP, int KW, int NV,
-    double sigma, float* pm,
-    unsigned* s_target, int* s_flag) {
-    float* stage = pm;                                // [KMAX][CHV] slab columns of a chunk (TMA, 128-byte aligned)
-    float* Arow = stage + KMAX * CHV;                 // [CHV][KW] rows of the chunk's active voxels
-    float* s_ch = Arow + CHV * KW;                    // [CHV] their change of h
-    float* s_cp = s_ch + CHV;                         // [CHV] their pi
-    float* s_ho = s_cp + CHV;                         // [CHV] their previous h (first evaluation after a new column)
-    int* s_dl = reinterpret_cast<int*>(s_ho + CHV);   // [CHV] slots of the rows whose h changed
-    __shared__ float s_zs[CHV], s_zc[CHV];
-    __shared__ unsigned s_bu[CHV / 32], s_bd[CHV / 32];
-    __shared__ float s_ga[PT], s_gna[PT], s_ea[PT];  // [lane set][column]
-    __shared__ int s_mode0;
-    __shared__ __align__(8) unsigned long long s_bars[NST_MAX];
-    __shared__ float s_yh[KMAX], s_yl[KMAX];
+    uint8_t* __restrict__ vstate, float* __restrict__ H_keep, bool nonneg, int bid, int G, int K, double sigma,
+    float* ring_mem, unsigned* s_target, int* s_flag) {
+    // the step's memory; its H holds rows of changed voxels between steps
+    __shared__ StepMem sm;
+    __shared__ StepState ss;
+    __shared__ __align__(16) float2 s_y[KMAX];
     __shared__ StructTermsF s_tf[SMAX];
-    __shared__ float s_red[PW];
-    __shared__ float s_scr[8 * 24];
-    __shared__ int s_last, s_stop;
+    __shared__ float2 s_al[PW][32];  // a tile's active voxels: pi (EXT: h times the new column's dose), offset in a group
+    __shared__ float s_red[2][PW];
+    // a warp's list: the changed voxels, their change of h and their row of the
+    // pool; then the warps' gradient sums
+    __shared__ __align__(16) int s_dj[PW][LIST];
+    __shared__ __align__(16) float s_dh[PW][LIST];
+    __shared__ unsigned char s_ds[PW][LIST];
+    __shared__ float s_ch[HB];  // change of h of the rows in hand
+    __shared__ int s_row[HB];   // their rows of A
+    __shared__ int s_nd[PW];
+    __shared__ int s_mode0, s_pool, s_lost;
+    float(*A)[H_LD] = sm.H;
+    float(*s_g)[KMAX] = reinterpret_cast<float(*)[KMAX]>(&s_dj[0][0]);    // g or the new column of H
+    float(*s_gn)[KMAX] = reinterpret_cast<float(*)[KMAX]>(&s_dh[0][0]);  // gn
+    static_assert(KMAX <= LIST && HB <= KMAX && HB < 256, "scratch fits");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned lt = (1u << lane) - 1u;
     for (int i = tid; i < S; i += PT) s_tf[i] = tf[i];
-    const int KB = KP / 4;
+    const int KP = (K + 3) / 4 * 4;
+    // update of H: thread (eb, vl) the 2x2 blocks eb, eb + PT / NV, ... of the upper
+    // triangle over every NV-th row
+    const int NV = persist_lanes(K);
+    const int KB = KP / 2;
     const int nb = KB * (KB + 1) / 2;
-    int rb = -1, cb = -1;
     const int vl = tid % NV;
-    if (tid < nb * NV) block_of(tid / NV, KB, rb, cb);
+    int rb0 = 0, cb0 = 0;
+    if (tid / NV < nb) block_of(tid / NV, KB, rb0, cb0);
+    // gradient: lane (vs, gl) takes the column group gl of every (32 / LP)-th active voxel
+    const int KG = KP / 4;
+    const int LP = KG <= 1 ? 1 : KG <= 2 ? 2 : KG <= 4 ? 4 : KG <= 8 ? 8 : 16;
+    const int gl = lane & (LP - 1), vs = lane / LP;
+    // tile i of this warp: bid + G (warp + PW i); warp 0 has the most
     const int n32 = (V + 31) / 32;
-    const int tiles_b = bid < n32 ? (n32 - 1 - bid) / G + 1 : 0;
-    // the block's chunks: bid, bid + G, bid + 2G, ...
-    const int n_ch = (V + CHV - 1) / CHV;
-    const int chunks_b = bid < n_ch ? (n_ch - 1 - bid) / G + 1 : 0;
-    auto chunk_of = [&](int m) { return bid + m * G; };
-    // copies in flight: nst stages of nbox boxes each, copy n (n = 0, 1, ... over
-    // the launch) holding position n mod chunks_b in stage n mod nst
-    // a copy: KP / 16 boxes of 16 columns, then (KP mod 16) / 4 of 4 columns
-    const int nbox = KP / BOXC, nbox4 = (KP % BOXC) / 4;
-    const int nst = max(1, min(NST_MAX, KMAX / KP));
-    const int stage_floats = KP * CHV;
-    int n_use = 0, n_iss = 0;  // copies consumed (every thread), issued (thread 0)
-    bool lost = false;
-    // z by column halves: thread (half, v), columns [k0h, k1h); g by column kq
-    // and lane set ls (PT / KP lane sets: the fewer the columns, the more rows
-    // each column's sums are split over)
-    const int half = tid / CHV, v = tid % CHV;
-    const int KH = KP / 8 * 4;
-    const int k0h = half ? KH : 0, k1h = half ? KP : KH;
-    const int nls = PT / KP;
-    const int kq = tid % KP, ls = tid / KP;
+    const int rounds = bid < n32 ? (n32 - 1 - bid) / (PW * G) + 1 : 0;
+    TileRing ring;
+    ring.init(ring_mem + warp * (RING * RING_LD), slab, ld, KG, bid + G * warp, PW * G, n32);
+    const float4* y4 = reinterpret_cast<const float4*>(s_y);
     int n_ev = 0;  // evaluations of this solve so far
-    auto issue = [&](int n) {  // thread 0
-        const int sidx = n % nst;
-        float* dst = stage + sidx * stage_floats;
-        mbar_expect_tx(&s_bars[sidx], (unsigned)(stage_floats * sizeof(float)));
-        const int c = chunk_of(n % chunks_b);
-        for (int q = 0; q < nbox; ++q) tma_load_2d(dst + q * BOXC * CHV, tmap, c * CHV, q * BOXC, &s_bars[sidx]);
-        for (int q = 0; q < nbox4; ++q)
-            tma_load_2d(dst + (nbox * BOXC + 4 * q) * CHV, tmap + 1, c * CHV, nbox * BOXC + 4 * q, &s_bars[sidx]);
-    };
-    // warm start (every block computes it; block 0 also writes the solver
-    // state): the previous optimum, the new aperture K - 1 at 0
+    const unsigned tag0 = __ldcg(&st->epoch);  // evaluations of the plan before this solve
+    // warm start (every block): the previous optimum, the new aperture K - 1 at 0
     if (tid < KMAX) {
         const double yv = tid < K - 1 ? __ldcg(&st->y[tid]) : 0.0;
-        const float hi = (float)yv;
-        s_yh[tid] = hi;
-        s_yl[tid] = (float)(yv - (double)hi);
-        if (bid == 0 && tid < K) {
-            st->yt[tid] = yv;
-            st->d[tid] = 0.0;
-        }
+        ss.y[tid] = yv;
+        ss.yt[tid] = yv;
+        ss.d[tid] = 0.0;
+        ss.g[tid] = 0.0;
     }
-    if (bid == 0 && tid == 0) {
-        st->K = K;
-        st->iter = 0;
-        st->phase = 0;
-        st->done = 0;
-        st->status = MASTER_RUNNING;
-        st->alpha = 1.0;
-        st->n_eval = 0;
-        st->err = 0;
-        st->ticket = 0;
-        st->final_pending = 0;
-    }
-    if (tid < NST_MAX) mbar_init(&s_bars[tid], 1);
-    if (tid == 0) {  // the kept partial H: extend it by the new column, keep it, or rebuild it
+    if (tid == 0) {
+        ss.F = 0.0;
+        ss.alpha = 1.0;
+        ss.tol = 0.0;
+        ss.res = 0.0;
+        ss.iter = ss.phase = ss.done = ss.n_eval = ss.final_pending = 0;
+        ss.status = MASTER_RUNNING;
+        s_pool = 0;
+        s_lost = 0;
+        // the kept partial H: extended by the new column, kept, or rebuilt
         const int iG = __ldcg(&st->inc_G), iK = __ldcg(&st->inc_K);
         s_mode0 = iG == G && iK == K - 1 ? MODE_EXT : iG == G && iK == K ? MODE_INC : MODE_FULL;
+        if (bid == 0) {  // a solve that ends early leaves these
+            st->K = K;
+            st->done = 0;
+            st->status = MASTER_RUNNING;
+            st->err = 0;
+        }
     }
     __syncthreads();
-    if (tid == 0 && chunks_b > 0)  // the first nst copies; the slab does not change during the solve
-        for (; n_iss < nst; ++n_iss) issue(n_iss);
-    const int mode0 = s_mode0;
-    bool first = true;
+    bool broken = false;
     for (;;) {
-        if (!first) {  // the state of the previous step (all blocks read it after the barrier)
-            if (tid == 0) s_stop = __ldcg(&st->done) | __ldcg(&st->err);
-            if (tid < KMAX) {
-                const double yv = tid < K ? __ldcg(&st->yt[tid]) : 0.0;
-                const float hi = (float)yv;
-                s_yh[tid] = hi;
-                s_yl[tid] = (float)(yv - (double)hi);
-            }
-            __syncthreads();
-            if (s_stop) break;
+        if (tid < KMAX) {
+            const double yv = tid < K ? ss.yt[tid] : 0.0;
+            const float hi = (float)yv;
+            s_y[tid] = make_float2(hi, (float)(yv - (double)hi));
         }
-        first = false;
-        // ---- A. the block's chunks of CHV voxels in turn.  The chunk's slab
-        // columns arrive in a stage buffer ([16 q][CHV] per box of 16 columns,
-        // TMA, copies in flight ahead).  Per chunk:
-        //   z: thread (half, v) takes the compensated products of voxel v over
-        //      its half of the columns (four chains); half 1 hands its pair to
-        //      half 0, which forms z, pi, h, F and the voxel's curvature state;
-        //   rows: the rows of the voxels with h > 0 now or at the previous
-        //      evaluation go, compacted, to Arow (each half copies its own
-        //      columns), with pi, the change of h and (first evaluation after a
-        //      new column) the previous h; then the next copy is issued;
-        //   every thread folds the rows in: g, the rounding scale of g and the
-        //      new column's curvature row by column (four lane sets), and the
-        //      change of H by 4x4 blocks over the rows whose h changed.
-        // The block's partial H is kept from one evaluation to the next (it is
-        // updated by the changes of h only); the first evaluation of a solve
-        // extends it by the new column, or rebuilds it when it is not valid.
-        const int mode = n_ev == 0 ? mode0 : MODE_INC;
-        float facc = 0.f;
-        float hs[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) hs[q] = 0.f;
-        float ga = 0.f, gna = 0.f, ea = 0.f;
-        int nd_blk = 0;  // rows of the block whose h changed (uniform)
-        // the voxel's label and curvature state, one chunk ahead (their latency
-        // passes behind the previous chunk's work)
-        auto voxel_in = [&](int m, int& lab_, unsigned& osv_) {
-            const int jj = chunk_of(m) * CHV + v;
-            const bool own = !half && m < chunks_b && jj < V;
-            lab_ = own && S >= 0 ? (int)vstruct[jj] : 0;
-            osv_ = own && mode != MODE_FULL ? (unsigned)vstate[jj] : 0u;
+        __syncthreads();
+        // ---- A. the warp's tiles
+        const int mode = n_ev == 0 ? s_mode0 : MODE_INC;
+        float facc = 0.f, gk = 0.f, gnk = 0.f;
+        float4 ga = make_float4(0.f, 0.f, 0.f, 0.f), gna = ga;  // EXT: ga holds the new column of H
+        int nd_w = 0;           // voxels in the warp's list
+        bool h_written = false;
+        // the lane's voxel of tile i: its label and curvature state, and its dose at
+        // the last evaluation (EXT: its pi), requested one tile ahead
+        auto voxel_in = [&](int i, int& lab_, unsigned& osv_, float& x_) {
+            const int jj = (bid + G * (warp + PW * i)) * 32 + lane;
+            const bool in = i < ring.tiles && jj < V;
+            lab_ = in && S >= 0 ? (int)vstruct[jj] : 0;
+            osv_ = in && mode != MODE_FULL ? (unsigned)vstate[jj] : 0u;
+            x_ = in && mode != MODE_FULL ? __ldcg((mode == MODE_EXT ? pi_out : z_out) + jj) : 0.f;
         };
-        int lab_n = 0;
-        unsigned osv_n = 0u;
-        voxel_in(0, lab_n, osv_n);
-        for (int m = 0; m < chunks_b && !lost; ++m) {
-            const int sidx = n_use % nst;
-            const float* stage_c = stage + sidx * stage_floats;
-            const int j = chunk_of(m) * CHV + v;
+        int lab_n;
+        unsigned osv_n;
+        float x_n;
+        voxel_in(0, lab_n, osv_n, x_n);
+        // adds the n_a listed voxels of the tile in use: their doses times the listed
+        // value to ga (and the product of the magnitudes to gna)
+        auto add_rows = [&](int n_a, bool scale_too) {
+            if (gl < KG) {
+                const float* base = ring.group(gl);
+                for (int r = vs; r < n_a; r += 32 / LP) {
+                    const float2 e = s_al[warp][r];
+                    const float4 a = *reinterpret_cast<const float4*>(base + __float_as_int(e.y));
+                    ga.x = fmaf(a.x, e.x, ga.x);
+                    ga.y = fmaf(a.y, e.x, ga.y);
+                    ga.z = fmaf(a.z, e.x, ga.z);
+                    ga.w = fmaf(a.w, e.x, ga.w);
+                    if (scale_too) {
+                        const float pa = fabsf(e.x);
+                        gna.x = fmaf(fabsf(a.x), pa, gna.x);
+                        gna.y = fmaf(fabsf(a.y), pa, gna.y);
+                        gna.z = fmaf(fabsf(a.z), pa, gna.z);
+                        gna.w = fmaf(fabsf(a.w), pa, gna.w);
+                    }
+                }
+            }
+        };
+        for (int i = 0; i < rounds; ++i) {
+            const bool mine = i < ring.tiles;
+            const int j = (bid + G * (warp + PW * i)) * 32 + lane;
             const int lab = lab_n;
             const unsigned osv = osv_n;
-            voxel_in(m + 1, lab_n, osv_n);
-            const bool got = mbar_wait(&s_bars[sidx], (unsigned)((n_use / nst) & 1));
-            float sc[4] = {0.f, 0.f, 0.f, 0.f}, cc[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int k = k0h; k < k1h; k += 4) {  // columns K..KP-1 are zero and meet y = 0
-                dot2_step(sc[0], cc[0], stage_c[k * CHV + v], s_yh[k], s_yl[k]);
-                dot2_step(sc[1], cc[1], stage_c[(k + 1) * CHV + v], s_yh[k + 1], s_yl[k + 1]);
-                dot2_step(sc[2], cc[2], stage_c[(k + 2) * CHV + v], s_yh[k + 2], s_yl[k + 2]);
-                dot2_step(sc[3], cc[3], stage_c[(k + 3) * CHV + v], s_yh[k + 3], s_yl[k + 3]);
-            }
-            float s = sc[0], c = cc[0];
-#pragma unroll
-            for (int q = 1; q < 4; ++q) {
-                const float t2 = s + sc[q];
-                const float bb = t2 - s;
-                const float e = (s - (t2 - bb)) + (sc[q] - bb);
-                s = t2;
-                c += e + cc[q];
-            }
-            if (half) {
-                s_zs[v] = s;
-                s_zc[v] = c;
-            }
-            if (__syncthreads_or(!got)) {  // a copy never arrived: stop issuing, report it
-                lost = true;
-                break;
-            }
-            float p = 0.f, dh = 0.f, hold = 0.f;
-            bool uni = false;
-            if (!half) {
-                {  // TwoSum of the halves' sums
-                    const float s1 = s_zs[v];
-                    const float t2 = s + s1;
-                    const float bb = t2 - s;
-                    const float e = (s - (t2 - bb)) + (s1 - bb);
-                    s = t2;
-                    c += e + s_zc[v];
-                }
-                float h = 0.f;
+            const float x_in = x_n;
+            voxel_in(i + 1, lab_n, osv_n, x_n);
+            if (mine && mode == MODE_EXT) {
+                ring.wait();
+                float hs = 0.f;
                 if (j < V) {
-                    const StructTermsF t = S >= 0 ? s_tf[lab] : voxel_terms(tf, j);
-                    const float du = (t.tu - s) - c;
-                    const float dov = (s - t.to) + c;
+                    const StructTermsF tt = S >= 0 ? s_tf[lab] : voxel_terms(tf, j);
+                    const float a = ring.group(KG - 1)[4 * lane + ((K - 1) & 3)];
+                    hs = 2.f * (((osv & 1u) ? tt.a : 0.f) + ((osv & 2u) ? tt.b : 0.f)) * a;
+                    gk = fmaf(a, x_in, gk);
+                    gnk = fmaf(fabsf(a), fabsf(x_in), gnk);
+                }
+                const unsigned am = __ballot_sync(FULL, hs != 0.f);
+                if (hs != 0.f) s_al[warp][__popc(am & lt)] = make_float2(hs, __int_as_float(4 * lane));
+                __syncwarp();
+                add_rows(__popc(am), false);
+                ring.release();
+            } else if (mine) {
+                ring.wait();
+                auto dose4 = [&](int k) { return *reinterpret_cast<const float4*>(ring.group(k >> 2) + 4 * lane); };
+                float s = 0.f, c = 0.f;
+                const bool fast = nonneg && mode != MODE_FULL && voxel_dot_biased(KP, y4, x_in, s, c, dose4);
+                if (__any_sync(FULL, !fast && j < V)) {
+                    float s2, c2;
+                    voxel_dot(KP, y4, s2, c2, dose4);
+                    if (!fast) {
+                        s = s2;
+                        c = c2;
+                    }
+                }
+                float p = 0.f, h = 0.f, dh = 0.f;
+                if (j < V) {
+                    const StructTermsF tt = S >= 0 ? s_tf[lab] : voxel_terms(tf, j);
+                    const float du = (tt.tu - s) - c;
+                    const float dov = (s - tt.to) + c;
                     const float u = fmaxf(du, 0.f), o = fmaxf(dov, 0.f);
-                    p = 2.f * (t.b * o - t.a * u);
-                    h = 2.f * ((du > 0.f ? t.a : 0.f) + (dov > 0.f ? t.b : 0.f));
-                    facc = fmaf(t.a * u, u, fmaf(t.b * o, o, facc));
+                    p = 2.f * (tt.b * o - tt.a * u);
+                    h = 2.f * ((du > 0.f ? tt.a : 0.f) + (dov > 0.f ? tt.b : 0.f));
+                    facc = fmaf(tt.a * u, u, fmaf(tt.b * o, o, facc));
                     z_out[j] = s + c;  // the state of the round when this point is the final one
                     pi_out[j] = p;
                     const unsigned nsv = (du > 0.f ? 1u : 0u) | (dov > 0.f ? 2u : 0u);
-                    hold = 2.f * (((osv & 1u) ? t.a : 0.f) + ((osv & 2u) ? t.b : 0.f));
-                    dh = h - hold;
+                    dh = h - 2.f * (((osv & 1u) ? tt.a : 0.f) + ((osv & 2u) ? tt.b : 0.f));
                     if (nsv != osv || mode == MODE_FULL) vstate[j] = (uint8_t)nsv;
                 }
-                uni = h > 0.f || hold > 0.f;
-                const unsigned bu = __ballot_sync(FULL, uni);
-                const unsigned bd = __ballot_sync(FULL, uni && dh != 0.f);
-                if (lane == 0) {
-                    s_bu[warp] = bu;
-                    s_bd[warp] = bd;
-                }
-            }
-            __syncthreads();
-            int n_u = 0, base = 0, n_d = 0, based = 0;
-            const int wv = v >> 5;  // the voxel's warp in half 0
-#pragma unroll
-            for (int w = 0; w < CHV / 32; ++w) {
-                const int cu = __popc(s_bu[w]), cd = __popc(s_bd[w]);
-                base += w < wv ? cu : 0;
-                based += w < wv ? cd : 0;
-                n_u += cu;
-                n_d += cd;
-            }
-            const unsigned lt = (1u << lane) - 1u;
-            if ((s_bu[wv] >> lane) & 1u) {
-                const int slot = base + __popc(s_bu[wv] & lt);
-                float4* dst = reinterpret_cast<float4*>(Arow + slot * KW);
-                for (int q = k0h / 4; q < k1h / 4; ++q)
-                    dst[q] = make_float4(stage_c[(4 * q) * CHV + v], stage_c[(4 * q + 1) * CHV + v],
-                                         stage_c[(4 * q + 2) * CHV + v], stage_c[(4 * q + 3) * CHV + v]);
-                if (!half) {
-                    s_cp[slot] = p;
-                    s_ch[slot] = dh;
-                    s_ho[slot] = mode == MODE_EXT ? hold : 0.f;
-                    if ((s_bd[wv] >> lane) & 1u) s_dl[based + __popc(s_bd[wv] & lt)] = slot;
-                }
-            }
-            __syncthreads();  // the stage is free, the chunk's rows are in Arow
-            if (tid == 0) issue(n_iss++);  // copy n_use + nst into the freed stage
-            ++n_use;
-            nd_blk += n_d;
-            // g, the rounding scale of g and the new column's curvature row
-            if (kq < K && ls < nls) {
-                if (mode == MODE_EXT) {
-                    for (int i = ls; i < n_u; i += nls) {
-                        const float a = Arow[i * KW + kq], pv = s_cp[i];
-                        ga = fmaf(a, pv, ga);
-                        gna = fmaf(fabsf(a), fabsf(pv), gna);
-                        ea = fmaf(a * s_ho[i], Arow[i * KW + K - 1], ea);
+                const unsigned am = __ballot_sync(FULL, h > 0.f);
+                const unsigned dm = __ballot_sync(FULL, dh != 0.f);
+                if (h > 0.f) s_al[warp][__popc(am & lt)] = make_float2(p, __int_as_float(4 * lane));
+                if (dm) {
+                    int slot0 = HB;
+                    if (mode != MODE_FULL) {  // rows of the pool, in any order: the list gives the order of the sums
+                        if (lane == 0) slot0 = min(atomicAdd(&s_pool, __popc(dm)), HB);
+                        slot0 = __shfl_sync(FULL, slot0, 0);
                     }
-                } else {
-                    for (int i = ls; i < n_u; i += nls) {
-                        const float a = Arow[i * KW + kq], pv = s_cp[i];
-                        ga = fmaf(a, pv, ga);
-                        gna = fmaf(fabsf(a), fabsf(pv), gna);
+                    if (dh != 0.f) {
+                        const int r = __popc(dm & lt);
+                        s_dj[warp][nd_w + r] = j;
+                        s_dh[warp][nd_w + r] = dh;
+                        s_ds[warp][nd_w + r] = (unsigned char)min(slot0 + r, HB);
+                    }
+                    nd_w += __popc(dm);
+                    for (unsigned m = dm; m && slot0 < HB; m &= m - 1u, ++slot0) {
+                        if (lane < KG)
+                            *reinterpret_cast<float4*>(&A[slot0][4 * lane]) =
+                                *reinterpret_cast<const float4*>(ring.group(lane) + 4 * (__ffs(m) - 1));
                     }
                 }
+                __syncwarp();
+                add_rows(__popc(am), true);
+                ring.release();
             }
-            // the change of H over the rows whose h changed
-            if (rb >= 0) {
-                for (int ii = vl; ii < n_d; ii += NV) {
-                    const int i = s_dl[ii];
-                    const float4 ra = *reinterpret_cast<const float4*>(Arow + i * KW + 4 * rb);
-                    const float4 rc = *reinterpret_cast<const float4*>(Arow + i * KW + 4 * cb);
-                    const float hv = s_ch[i];
-                    const float a0 = ra.x * hv, a1 = ra.y * hv, a2 = ra.z * hv, a3 = ra.w * hv;
-                    hs[0] = fmaf(a0, rc.x, hs[0]);
-                    hs[1] = fmaf(a0, rc.y, hs[1]);
-                    hs[2] = fmaf(a0, rc.z, hs[2]);
-                    hs[3] = fmaf(a0, rc.w, hs[3]);
-                    hs[4] = fmaf(a1, rc.x, hs[4]);
-                    hs[5] = fmaf(a1, rc.y, hs[5]);
-                    hs[6] = fmaf(a1, rc.z, hs[6]);
-                    hs[7] = fmaf(a1, rc.w, hs[7]);
-                    hs[8] = fmaf(a2, rc.x, hs[8]);
-                    hs[9] = fmaf(a2, rc.y, hs[9]);
-                    hs[10] = fmaf(a2, rc.z, hs[10]);
-                    hs[11] = fmaf(a2, rc.w, hs[11]);
-                    hs[12] = fmaf(a3, rc.x, hs[12]);
-                    hs[13] = fmaf(a3, rc.y, hs[13]);
-                    hs[14] = fmaf(a3, rc.z, hs[14]);
-                    hs[15] = fmaf(a3, rc.w, hs[15]);
+            if (mode == MODE_EXT) continue;
+            // the listed changes into the kept partial H: once, after the last tile,
+            // unless a list could overflow before
+            const bool end = i == rounds - 1;
+            if (!end && (i < LIST / 32 - 1 || !__syncthreads_or(nd_w > LIST - 32))) continue;
+            if (lane == 0) s_nd[warp] = nd_w;
+            const bool any = __syncthreads_or(nd_w > 0) != 0;
+            nd_w = 0;
+            const bool rebuild = mode == MODE_FULL && !h_written;
+            if (!any && !rebuild) continue;
+            h_written = true;
+            int n_d = 0;
+#pragma unroll
+            for (int w = 0; w < PW; ++w) n_d += s_nd[w];
+            const bool pooled = mode != MODE_FULL && n_d <= HB;  // every row is in the pool
+            for (int eb = tid / NV; eb - tid / NV < nb; eb += PT / NV) {  // (uniform count: barriers inside)
+                const bool act = eb < nb;
+                int rb = rb0, cb = cb0;
+                if (act && eb >= PT / NV) block_of(eb, KB, rb, cb);
+                rb *= 2;
+                cb *= 2;
+                // entries (rb, cb), (rb, cb + 1), (rb + 1, cb), (rb + 1, cb + 1): those of the
+                // upper triangle, requested before the rows are summed
+                const bool wr = act && vl == 0;
+                float* keep = H_keep + (size_t)bid * HSTRIDE;
+                const bool e0 = wr && cb < K, e1 = wr && cb + 1 < K, e2 = e0 && rb < cb, e3 = e1;
+                const int i0 = tri_index(rb, cb, K), i1 = tri_index(rb, cb + 1, K);
+                float old[4] = {0.f, 0.f, 0.f, 0.f};
+                if (!rebuild) {
+                    if (e0) old[0] = keep[i0];
+                    if (e1) old[1] = keep[i1];
+                    if (e2) old[2] = keep[i0 + 1];
+                    if (e3) old[3] = keep[i1 + 1];
                 }
-            }
-            // Arow and the lists are next written after the next chunk's first two
-            // barriers, which every thread reaches only when done with this chunk
-        }
-        ++n_ev;
-        // ---- the block's partials: F; g, the rounding scale of g and the new
-        // column's curvature row (lane sets added in order); H in place
-        const float fw = warp_sum_f32(facc);
-        if (lane == 0) s_red[warp] = fw;
-        if (ls < nls) {
-            s_ga[ls * KP + kq] = ga;
-            s_gna[ls * KP + kq] = gna;
-            s_ea[ls * KP + kq] = ea;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double t = 0.0;
-            for (int w = 0; w < PW; ++w) t += (double)s_red[w];
-            F_part[bid] = t;
-            if (lost) st->err = 1;  // the step stops the solve at the last accepted point
-        }
-        if (tid < K) {
-            float g4 = 0.f, gn4 = 0.f, ext = 0.f;  // lane sets in order
-            for (int l = 0; l < nls; ++l) {
-                g4 += s_ga[l * KP + tid];
-                gn4 += s_gna[l * KP + tid];
-                ext += s_ea[l * KP + tid];
-            }
-            g_part[(size_t)tid * GS + bid] = (double)g4;
-            gn_part[(size_t)tid * GS + bid] = gn4;
-            if (mode == MODE_EXT) {
-                H_keep[(size_t)bid * HSTRIDE + tri_index(tid, K - 1, K)] = ext;
-                if (nd_blk == 0) H_part[(size_t)tri_index(tid, K - 1, K) * GS + bid] = ext;
-            }
-        }
-        __syncthreads();  // the new column's row is in place before the changes are added
-        if (mode == MODE_FULL || nd_blk > 0) {
-            const int span = NV < 32 ? NV : 32;
-            for (int o = span / 2; o > 0; o >>= 1)
-#pragma unroll
-                for (int q = 0; q < 16; ++q) hs[q] += __shfl_xor_sync(FULL, hs[q], o);
-            if (NV > 32 && lane == 0)
-#pragma unroll
-                for (int q = 0; q < 16; ++q) s_scr[warp * 24 + q] = hs[q];
-            __syncthreads();
-            if ((tid % NV) == 0 && tid < nb * NV) {
-                if (NV > 32) {
-                    const int w0 = tid >> 5, nw = NV >> 5;
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        float t = 0.f;
-                        for (int w = 0; w < nw; ++w) t += s_scr[(w0 + w) * 24 + q];
-                        hs[q] = t;
-                    }
-                }
-                float old[16];
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int r = 4 * rb + q, cl = 4 * cb + e;
-                        old[q * 4 + e] = mode != MODE_FULL && r < K && cl < K && r <= cl
-                                             ? H_keep[(size_t)bid * HSTRIDE + tri_index(r, cl, K)]
-                                             : 0.f;
-                    }
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int r = 4 * rb + q, cl = 4 * cb + e;
-                        if (r < K && cl < K && r <= cl) {
-                            const float nv = old[q * 4 + e] + hs[q * 4 + e];
-                            H_keep[(size_t)bid * HSTRIDE + tri_index(r, cl, K)] = nv;
-                            H_part[(size_t)tri_index(r, cl, K) * GS + bid] = nv;
+                float hs[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int r0 = 0; r0 < n_d; r0 += HB) {
+                    const int n = min(HB, n_d - r0);
+                    if (eb - tid / NV == 0 || n_d > HB) {  // the rows in hand: their change of h, their place in A
+                        __syncthreads();  // the rows before are summed
+                        if (tid < n || !pooled) {
+                            const int r = tid & (HB - 1);
+                            int w = 0, x = r0 + r;
+                            if (r < n) {
+                                while (x >= s_nd[w]) x -= s_nd[w++];
+                                if (tid < HB) {
+                                    s_ch[r] = s_dh[w][x];
+                                    s_row[r] = pooled ? (int)s_ds[w][x] : r;
+                                }
+                                if (!pooled) {
+                                    const float4* row = reinterpret_cast<const float4*>(slab) + s_dj[w][x];
+                                    for (int g = tid / HB; g < KG; g += PT / HB)
+                                        *reinterpret_cast<float4*>(&A[r][4 * g]) = __ldg(row + (size_t)g * ld);
+                                }
+                            }
                         }
+                        __syncthreads();
                     }
+                    if (act)
+                        for (int r = vl; r < n; r += NV) {
+                            const float* row = A[s_row[r]];
+                            const float2 ra = *reinterpret_cast<const float2*>(row + rb);
+                            const float2 rc = *reinterpret_cast<const float2*>(row + cb);
+                            const float hv = s_ch[r];
+                            const float a0 = ra.x * hv, a1 = ra.y * hv;
+                            hs[0] = fmaf(a0, rc.x, hs[0]);
+                            hs[1] = fmaf(a0, rc.y, hs[1]);
+                            hs[2] = fmaf(a1, rc.x, hs[2]);
+                            hs[3] = fmaf(a1, rc.y, hs[3]);
+                        }
+                }
+                for (int o = NV / 2; o > 0; o >>= 1)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) hs[q] += __shfl_xor_sync(FULL, hs[q], o);
+                auto put = [&](int idx, float v) {
+                    keep[idx] = v;
+                    H_part[(size_t)idx * GS + bid] = v;
+                };
+                if (e0) put(i0, old[0] + hs[0]);
+                if (e1) put(i1, old[1] + hs[1]);
+                if (e2) put(i0 + 1, old[2] + hs[2]);
+                if (e3) put(i1 + 1, old[3] + hs[3]);
+            }
+            if (tid == 0) s_pool = 0;
+            __syncthreads();  // the rows and lists are free
+        }
+        if (rounds == 0 && mode == MODE_FULL)  // a block without voxels: its part of H is 0
+            for (int e = tid; e < K * (K + 1) / 2; e += PT) {
+                H_keep[(size_t)bid * HSTRIDE + e] = 0.f;
+                H_part[(size_t)e * GS + bid] = 0.f;
+            }
+        ++n_ev;
+        // ---- the block's partials: F; g and its rounding scale (or the new
+        // aperture's, and its column of H), the warps in order
+        const float f0 = warp_sum_f32(mode == MODE_EXT ? gk : facc);
+        if (lane == 0) s_red[0][warp] = f0;
+        if (mode == MODE_EXT) {
+            const float f1 = warp_sum_f32(gnk);
+            if (lane == 0) s_red[1][warp] = f1;
+        }
+        for (int o = LP; o < 32; o <<= 1) {
+            ga.x += __shfl_xor_sync(FULL, ga.x, o);
+            ga.y += __shfl_xor_sync(FULL, ga.y, o);
+            ga.z += __shfl_xor_sync(FULL, ga.z, o);
+            ga.w += __shfl_xor_sync(FULL, ga.w, o);
+            gna.x += __shfl_xor_sync(FULL, gna.x, o);
+            gna.y += __shfl_xor_sync(FULL, gna.y, o);
+            gna.z += __shfl_xor_sync(FULL, gna.z, o);
+            gna.w += __shfl_xor_sync(FULL, gna.w, o);
+        }
+        if (lane < KG) {  // (lanes below LP)
+            *reinterpret_cast<float4*>(&s_g[warp][4 * lane]) = ga;
+            *reinterpret_cast<float4*>(&s_gn[warp][4 * lane]) = gna;
+        }
+        __syncthreads();
+        if (tid < 2 * KMAX) {  // g (or the new column of H), gn
+            const int k = tid & (KMAX - 1), a = tid / KMAX;
+            if (k < K) {
+                float x = 0.f;
+#pragma unroll
+                for (int w = 0; w < PW; ++w) x += a ? s_gn[w][k] : s_g[w][k];
+                if (mode == MODE_EXT) {
+                    if (a == 0) {
+                        H_keep[(size_t)bid * HSTRIDE + tri_index(k, K - 1, K)] = x;
+                        H_part[(size_t)tri_index(k, K - 1, K) * GS + bid] = x;
+                    }
+                } else if (a == 0) {
+                    g_part[(size_t)k * GS + bid] = (double)x;
+                } else {
+                    gn_part[(size_t)k * GS + bid] = x;
+                }
+            }
+        } else if (warp == PW - 1) {  // F in FP64 (or the new aperture's g and gn) over the warps
+            if (mode == MODE_EXT) {
+                float x = lane < PW ? s_red[0][lane] : 0.f, y = lane < PW ? s_red[1][lane] : 0.f;
+                x = warp_sum_f32(x);
+                y = warp_sum_f32(y);
+                if (lane == 0) {
+                    g_part[(size_t)(K - 1) * GS + bid] = (double)x;
+                    gn_part[(size_t)(K - 1) * GS + bid] = y;
+                }
+            } else {
+                double x = lane < PW ? (double)s_red[0][lane] : 0.0;
+#pragma unroll
+                for (int o = PW / 2; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
+                if (lane == 0) F_part[bid] = x;
             }
         }
         if (!grid_sync(gb, G, s_target, s_flag)) {
-            if (tid == 0) st->err = 2;
+            broken = true;
             break;
         }
-        // ---- B. reduction by every block, the step by the last one to finish
-        master_reduce_part(H_part, g_part, gn_part, F_part, GS, G, G, K, st, bid, G);
-        __syncthreads();
-        if (tid == 0) s_last = atom_add_acq_rel_gpu(&st->ticket, 1u) == (unsigned)G - 1u;
-        __syncthreads();
-        if (s_last) {
-            if (tid == 0) st->ticket = 0;
-            master_step_body(st, max_iter, tol_rel, sigma);
+        // ---- B. reduction by every block
+        const unsigned tag = tag0 + (unsigned)n_ev;
+        master_reduce_words(H_part, g_part, gn_part, F_part, GS, G, K, st, bid, mode == MODE_EXT, tag);
+        // ---- C. the step, by every block on its own copy of the state.  Every
+        // word of this evaluation is waited for (EXT: those of variable K - 1; the
+        // others are the last evaluation's).
+        if (tid < STEP_T) {
+            const int v = tid & (KMAX - 1);
+            unsigned long long w[KMAX * KMAX / STEP_T], x[5];
+            auto waits = [&](int r) { return r < K && v <= r && (mode != MODE_EXT || r == K - 1); };
+            // first one word that the last reducing warps write, until it is there
+            // (every thread polling all its words would keep the L2 from the reducers)
+            int tries = 0;
+            auto again = [&]() {
+                if (++tries < GRID_WAIT_LIMIT && ((tries & 4095) || !ld_acquire_gpu(&gb->broken))) return true;
+                s_lost = 1;
+                return false;
+            };
+            const unsigned long long* probe = &st->wgn[K - 1];
+            while ((unsigned)(word_get(probe) >> 32) != tag && again()) __nanosleep(40);
+            for (bool ok = false; !ok;) {
+                ok = true;
+#pragma unroll
+                for (int m = 0; m < KMAX * KMAX / STEP_T; ++m) {
+                    const int r = 4 * m + (tid >> 6);
+                    if (r < K && v <= r) w[m] = word_get(&st->wH[r * KMAX + v]);
+                }
+                if (v < K) {
+                    x[0] = word_get(&st->wg[2 * v]);
+                    x[1] = word_get(&st->wg[2 * v + 1]);
+                    x[2] = word_get(&st->wgn[v]);
+                }
+                x[3] = word_get(&st->wF[0]);
+                x[4] = word_get(&st->wF[1]);
+#pragma unroll
+                for (int m = 0; m < KMAX * KMAX / STEP_T; ++m)
+                    if (waits(4 * m + (tid >> 6))) ok = ok && (unsigned)(w[m] >> 32) == tag;
+                if (v < K && (mode != MODE_EXT || v == K - 1))
+                    ok = ok && (unsigned)(x[0] >> 32) == tag && (unsigned)(x[1] >> 32) == tag &&
+                         (unsigned)(x[2] >> 32) == tag;
+                if (mode != MODE_EXT) ok = ok && (unsigned)(x[3] >> 32) == tag && (unsigned)(x[4] >> 32) == tag;
+                if (!ok && !again()) break;
+            }
+#pragma unroll
+            for (int m = 0; m < KMAX * KMAX / STEP_T; ++m) {
+                const int r = 4 * m + (tid >> 6);
+                if (r < K && v <= r) sm.H[r][v] = __uint_as_float((unsigned)w[m]);
+            }
+            step_sync();
+            if (!s_lost)
+                master_step_body<true>(&ss, K, words_f64(x[3], x[4]), v < K ? words_f64(x[0], x[1]) : 0.0,
+                                       v < K ? __uint_as_float((unsigned)x[2]) : 0.f, max_iter, tol_rel, sigma, sm);
         }
-        if (!grid_sync(gb, G, s_target, s_flag)) {
-            if (tid == 0) st->err = 2;
+        __syncthreads();
+        if (s_lost) {
+            if (tid == 0) atomicExch(&gb->broken, 1u);
+            broken = true;
             break;
         }
+        if (ss.done) break;
     }
-    if (tid == 0) {
-        // no copy of this block outlives the launch (a lost one is not waited for again)
-        for (int n = lost ? n_use + 1 : n_use; n < n_iss; ++n) mbar_wait(&s_bars[n % nst], (unsigned)((n / nst) & 1));
-        s_stop = __ldcg(&st->err) == 2;
-        if (bid == 0) {  // the kept partial H and voxel states are those of the last evaluation
-            st->inc_G = __ldcg(&st->err) == 0 ? G : 0;
+    copies_wait<0>();  // no copy outlives the launch
+    if (broken) {      // a wait ran out: the host reports it
+        if (tid == 0) {
+            st->err = 2;
+            if (bid == 0) {
+                st->inc_G = 0;
+                st->epoch = tag0 + (unsigned)n_ev + 1u;
+            }
+        }
+        return;
+    }
+    if (bid == 0) {  // the solver state, and the round's record
+        if (tid < K) {
+            st->y[tid] = ss.y[tid];
+            st->yt[tid] = ss.yt[tid];
+            st->d[tid] = ss.d[tid];
+            st->g[tid] = ss.g[tid];
+        }
+        if (tid == 0) {
+            st->F = ss.F;
+            st->alpha = ss.alpha;
+            st->tol = ss.tol;
+            st->res = ss.res;
+            st->iter = ss.iter;
+            st->phase = ss.phase;
+            st->status = ss.status;
+            st->n_eval = ss.n_eval;
+            st->ticket = 0;
+            st->final_pending = ss.final_pending;
+            st->epoch = tag0 + (unsigned)n_ev;
+            // the kept partial H, the voxel states, z, pi and the reduced sums are
+            // those of the last evaluation: of the accepted point, or not kept
+            st->inc_G = ss.final_pending ? 0 : G;
             st->inc_K = K;
+            st->done = 1;
+            if (cg != nullptr) {
+                cg->trace[K - 1] = ss.F;
+                cg->res[K - 1] = ss.res;
+                cg->tol[K - 1] = ss.tol;
+                cg->evals[K - 1] = ss.n_eval;
+                cg->status[K - 1] = ss.status;
+            }
         }
     }
-    __syncthreads();
-    if (s_stop) return;  // a barrier timed out: the host reports it
     // the solve stopped at an accepted point other than the last one evaluated:
     // z and pi of that point
-    if (__ldcg(&st->final_pending)) {
+    if (ss.final_pending) {
         if (tid < KMAX) {
-            const double yv = tid < K ? __ldcg(&st->y[tid]) : 0.0;
+            const double yv = tid < K ? ss.y[tid] : 0.0;
             const float hi = (float)yv;
-            s_yh[tid] = hi;
-            s_yl[tid] = (float)(yv - (double)hi);
+            s_y[tid] = make_float2(hi, (float)(yv - (double)hi));
         }
         __syncthreads();
-        for (int i = warp; i < tiles_b; i += PW) {
-            const int j = (bid + i * G) * 32 + lane;
-            const bool in = j < V;
-            float sc[4] = {0.f, 0.f, 0.f, 0.f}, cc[4] = {0.f, 0.f, 0.f, 0.f};
-            const float* col = slab + (in ? j : 0);
-            for (int k = 0; k < KP; k += 4) {
-                dot2_step(sc[0], cc[0], __ldcg(col + (size_t)k * ld), s_yh[k], s_yl[k]);
-                dot2_step(sc[1], cc[1], __ldcg(col + (size_t)(k + 1) * ld), s_yh[k + 1], s_yl[k + 1]);
-                dot2_step(sc[2], cc[2], __ldcg(col + (size_t)(k + 2) * ld), s_yh[k + 2], s_yl[k + 2]);
-                dot2_step(sc[3], cc[3], __ldcg(col + (size_t)(k + 3) * ld), s_yh[k + 3], s_yl[k + 3]);
-            }
-            float s = sc[0], c = cc[0];
-#pragma unroll
-            for (int q = 1; q < 4; ++q) {
-                const float t2 = s + sc[q];
-                const float bb = t2 - s;
-                const float e = (s - (t2 - bb)) + (sc[q] - bb);
-                s = t2;
-                c += e + cc[q];
-            }
-            if (in) {
-                const StructTermsF t = S >= 0 ? s_tf[vstruct[j]] : voxel_terms(tf, j);
-                const float u = fmaxf((t.tu - s) - c, 0.f), o = fmaxf((s - t.to) + c, 0.f);
+        for (int t = bid + G * warp; t < n32; t += PW * G) {
+            const int j = t * 32 + lane;
+            float s, c;
+            voxel_dot(KP, y4, s, c, [&](int k) {  // the slab's columns are padded past V
+                return __ldg(reinterpret_cast<const float4*>(slab) + (size_t)(k >> 2) * ld + j);
+            });
+            if (j < V) {
+                const StructTermsF tt = S >= 0 ? s_tf[vstruct[j]] : voxel_terms(tf, j);
+                const float u = fmaxf((tt.tu - s) - c, 0.f), o = fmaxf((s - tt.to) + c, 0.f);
                 z_out[j] = s + c;
-                pi_out[j] = 2.f * (t.b * o - t.a * u);
+                pi_out[j] = 2.f * (tt.b * o - tt.a * u);
             }
         }
-    }
-    if (cg != nullptr && bid == 0 && tid == 0) {  // the round's record
-        cg->trace[K - 1] = __ldcg(&st->F);
-        cg->res[K - 1] = __ldcg(&st->res);
-        cg->tol[K - 1] = __ldcg(&st->tol);
-        cg->evals[K - 1] = __ldcg(&st->n_eval);
-        cg->status[K - 1] = __ldcg(&st->status);
     }
 }
 
 
 template <bool BATCH>
-__global__ void __launch_bounds__(PT, 2) k_master_persist(const __grid_constant__ MasterTask t1,
-                                                          const MasterTask* __restrict__ tasks,
-                                                       int GB, int K, int KP, int KW, int NV, double sigma) {
-#define DAO_TASK(f) (BATCH ? tasks[blockIdx.x / GB].f : t1.f)
-    const float* __restrict__ slab = DAO_TASK(slab);
-    const int ld = DAO_TASK(ld), V = DAO_TASK(V), GS = DAO_TASK(GS), S = DAO_TASK(S), max_iter = DAO_TASK(max_iter);
-    const CUtensorMap* tmap = BATCH ? tasks[blockIdx.x / GB].tmap : t1.tmap;
-    MasterDev* __restrict__ st = DAO_TASK(st);
-    GridBar* __restrict__ gb = DAO_TASK(gb);
-    float* __restrict__ H_part = DAO_TASK(H_part);
-    double* __restrict__ g_part = DAO_TASK(g_part);
-    float* __restrict__ gn_part = DAO_TASK(gn_part);
-    double* __restrict__ F_part = DAO_TASK(F_part);
-    const uint8_t* __restrict__ vstruct = DAO_TASK(vstruct);
-    const StructTermsF* __restrict__ tf = DAO_TASK(tf);
-    const double tol_rel = DAO_TASK(tol_rel);
-    const int* __restrict__ skip = DAO_TASK(skip);
-    float* __restrict__ z_out = DAO_TASK(z_out);
-    float* __restrict__ pi_out = DAO_TASK(pi_out);
-    CGDev* __restrict__ cg = DAO_TASK(cg);
-    uint8_t* __restrict__ vstate = DAO_TASK(vstate);
-    float* __restrict__ H_keep = DAO_TASK(H_keep);
-#undef DAO_TASK
+__global__ void __launch_bounds__(PT, 1) k_master_persist(const __grid_constant__ MasterTask t1,
+                                                          const MasterTask* __restrict__ tasks, int GB, int K,
+                                                          double sigma) {
+    const MasterTask& t = BATCH ? tasks[blockIdx.x / GB] : t1;
     const int bid = BATCH ? (int)(blockIdx.x % GB) : (int)blockIdx.x;
-    if (K <= 0) {  // pool size from the device (one graph for every round); KW sets the layout below
-        K = __ldcg(&cg->K);
-        KP = (K + 3) / 4 * 4;
-        KW = master_kw(K);
-        NV = persist_lanes(K);
-    }
-    extern __shared__ __align__(128) float pm[];
+    extern __shared__ __align__(128) float ring_mem[];
     __shared__ int s_flag, s_stop0;
     __shared__ unsigned s_target;
+    const int* skip = t.skip;
     if (skip != nullptr && *skip) return;  // the same for every block
+    if (K <= 0) K = __ldcg(&t.cg->K);      // pool size from the device (one graph for every round)
     const int G = BATCH ? GB : (int)gridDim.x;
     if (threadIdx.x == 0) {  // barrier base; a solve whose barrier broke runs no further master solve
-        const unsigned c = *reinterpret_cast<volatile unsigned*>(&gb->count);
+        const unsigned c = *reinterpret_cast<volatile unsigned*>(&t.gb->count);
         s_target = c - c % (unsigned)G;
-        s_stop0 = *reinterpret_cast<volatile unsigned*>(&gb->broken) != 0;
+        s_stop0 = *reinterpret_cast<volatile unsigned*>(&t.gb->broken) != 0;
     }
     __syncthreads();
     if (s_stop0) return;
-    master_solve_group(slab, tmap, ld, V, GS, S, max_iter, st, gb, H_part, g_part, gn_part, F_part, vstruct, tf,
-                       tol_rel, z_out, pi_out, cg, vstate, H_keep, bid, G, K, KP, KW, NV, sigma, pm, &s_target,
-                       &s_flag);
+    master_solve_group(t.slab, t.ld, t.V, t.GS, t.S, t.max_iter, t.st, t.gb, t.H_part, t.g_part, t.gn_part, t.F_part,
+                       t.vstruct, t.tf, t.tol_rel, t.z_out, t.pi_out, t.cg, t.vstate, t.H_keep, t.nonneg != 0, bid, G, K, sigma,
+                       ring_mem, &s_target, &s_flag);
 }
-
 
 }  // namespace
 
@@ -1509,14 +1775,14 @@ size_t master_hess_smem(int K, int n_tiles) {
            2 * CH * sizeof(float);
 }
 
-// Voxel lanes per 4x4 block of H in the persistent solve: the most (a power of
-// two) for which every block of the triangle has its lanes among the 256 threads.
+// Row lanes per 2x2 block of H in the persistent solve: the most (a power of
+// two, within a warp) for which every block of the triangle has its lanes among
+// the threads.
 __host__ __device__ int persist_lanes(int K) {
-    const int KP = (K + 3) / 4 * 4;
-    const int KB = KP / 4;
+    const int KB = (K + 3) / 4 * 2;
     const int nb = KB * (KB + 1) / 2;
     int nv = 1;
-    while (nb > 0 && nv * 2 * nb <= PT) nv *= 2;
+    while (nb > 0 && nv < 32 && nv * 2 * nb <= PT) nv *= 2;
     return nv;
 }
 
@@ -1578,11 +1844,9 @@ cudaError_t master_configure() {
     cudaError_t e = cudaFuncSetAttribute(k_master_eval, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)master_eval_smem(KMAX));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_master_persist<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)PERSIST_SMEM_MAX);
+    e = cudaFuncSetAttribute(k_master_persist<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RING_BYTES);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_master_persist<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)PERSIST_SMEM_MAX);
+    e = cudaFuncSetAttribute(k_master_persist<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RING_BYTES);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_master_hess, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
@@ -1616,58 +1880,28 @@ cudaError_t launch_master_hess(const MasterBuffers& mb, int K, int mode, cudaStr
 cudaError_t launch_master_step(int K, const MasterBuffers& mb, int max_iter, double tol_rel,
                                cudaGraphConditionalHandle cond, int use_cond, cudaStream_t stream, int* launches) {
     const int outs = K * (K + 1) / 2 + 2 * K + 1;
-    k_master_reduce_step<<<(outs + STEP_W - 1) / STEP_W, STEP_T, 0, stream>>>(
+    k_master_reduce_step<<<(outs + STEP_T / 32 - 1) / (STEP_T / 32), STEP_T, 0, stream>>>(
         mb.H_part, mb.g_part, mb.gn_part, mb.F_part, mb.GH, mb.grid[K], mb.st, max_iter, tol_rel, 1e-4, cond,
         use_cond);
     ++*launches;
     return cudaGetLastError();
 }
 
-// Dynamic shared memory of the persistent solve, the same for every voxel count
-// and grid size: the TMA stage (KMAX columns of a chunk), the chunk's active
-// rows at the widest row stride, their h and pi.
-size_t master_persist_smem(int V, int G) {
-    (void)V;
-    (void)G;
-    return (size_t)KMAX * CHV * sizeof(float) + (size_t)CHV * master_kw(KMAX) * sizeof(float) +
-           4 * (size_t)CHV * sizeof(float);
-}
-
-// Co-resident blocks of the persistent solve: 2 per SM when they fit, else 1;
-// 0 when a cooperative launch is not possible.  want > 0: that many blocks, or
-// the least number whose per-block working set fits the shared memory, if
-// more (at most the full count).
+// Co-resident blocks of the persistent solve: one per SM, and no more than give
+// every warp a tile of 32 voxels (fewer blocks have fewer partials to reduce
+// and arrivals to wait for); 0 when a cooperative launch is not possible.
+// want > 0: that many blocks, at most one per SM.
 int master_persist_grid(int V, int num_sms, int want) {
-    int dev = 0, coop = 0;
+    int dev = 0, coop = 0, occ = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_master_persist<false>, PT, RING_BYTES) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
-    if (want > 0) {
-        int occ = 0;
-        for (int G = want; G <= 2 * num_sms; ++G) {
-            const size_t smem = master_persist_smem(V, G);
-            if (smem > PERSIST_SMEM_MAX) continue;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_master_persist<false>, PT, smem) != cudaSuccess) {
-                cudaGetLastError();
-                return 0;
-            }
-            if (occ >= 1 && G <= occ * num_sms) return G;
-        }
-    }
-    for (int per = 2; per >= 1; --per) {
-        const int G = per * num_sms;
-        const size_t smem = master_persist_smem(V, G);
-        if (smem > PERSIST_SMEM_MAX) continue;
-        int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_master_persist<false>, PT, smem) != cudaSuccess) {
-            cudaGetLastError();
-            continue;
-        }
-        if (occ >= per) return G;
-    }
-    return 0;
+    if (occ < 1) return 0;
+    const int need = (V + 32 * PW - 1) / (32 * PW);
+    return std::min(num_sms, want > 0 ? want : std::max(need, 1));
 }
 
 cudaError_t launch_master_persist(const MasterBuffers& mb, const float* slab, int ld, int V, int K,
@@ -1677,11 +1911,7 @@ cudaError_t launch_master_persist(const MasterBuffers& mb, const float* slab, in
     const int G = mb.GP;
     if (G < 1) return cudaErrorInvalidConfiguration;
     if (K <= 0 && cg == nullptr) return cudaErrorInvalidValue;
-    int KP = K > 0 ? (K + 3) / 4 * 4 : 0;
-    int KW = K > 0 ? master_kw(K) : 0, NV = K > 0 ? persist_lanes(K) : 0;
     MasterTask t{};
-    t.tmap[0] = mb.tmap_p[0];
-    t.tmap[1] = mb.tmap_p[1];
     t.vstate = mb.vstate;
     t.H_keep = mb.H_keep;
     t.slab = slab;
@@ -1703,15 +1933,15 @@ cudaError_t launch_master_persist(const MasterBuffers& mb, const float* slab, in
     t.z_out = z_out;
     t.pi_out = pi_out;
     t.cg = cg;
+    t.nonneg = mb.nonneg;
     const MasterTask* none = nullptr;
     int GB = 0;
     double sigma = 1e-4;
-    void* args[] = {(void*)&t, (void*)&none, (void*)&GB, (void*)&K, (void*)&KP, (void*)&KW, (void*)&NV,
-                    (void*)&sigma};
+    void* args[] = {(void*)&t, (void*)&none, (void*)&GB, (void*)&K, (void*)&sigma};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(G);
     cfg.blockDim = dim3(PT);
-    cfg.dynamicSmemBytes = master_persist_smem(V, G);
+    cfg.dynamicSmemBytes = RING_BYTES;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -1724,38 +1954,42 @@ cudaError_t launch_master_persist(const MasterBuffers& mb, const float* slab, in
 }
 
 int master_batch_group(int n_tasks, int num_sms) {
-    // two co-resident blocks per SM (the shared memory per block is capped)
+    // one co-resident block per SM shared out evenly; more plans than SMs (up to
+    // two per SM) run one block each, in two launches
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_master_persist<true>, PT, master_persist_smem(0, 0)) !=
-        cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_master_persist<true>, PT, RING_BYTES) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
-    occ = std::min(occ, 2);
-    return n_tasks > 0 ? occ * num_sms / n_tasks : 0;
+    if (occ < 1 || n_tasks < 1 || n_tasks > 2 * num_sms) return 0;
+    return std::max(1, num_sms / n_tasks);
 }
 
-cudaError_t launch_master_persist_batch(const MasterTask* tasks, int n_tasks, int GB, int max_V, cudaStream_t stream,
-                                        int* launches) {
-    if (n_tasks < 1 || GB < 1) return cudaErrorInvalidConfiguration;
-    int K = 0, KP = 0, KW = 0, NV = 0;  // each group reads its pool size from its plan's device state
+cudaError_t launch_master_persist_batch(const MasterTask* tasks, int n_tasks, int GB, int num_sms,
+                                        cudaStream_t stream, int* launches) {
+    if (n_tasks < 1 || GB < 1 || GB > num_sms) return cudaErrorInvalidConfiguration;
+    int K = 0;  // each group reads its pool size from its plan's device state
     MasterTask none{};
     double sigma = 1e-4;
-    void* args[] = {(void*)&none, (void*)&tasks, (void*)&GB, (void*)&K, (void*)&KP, (void*)&KW, (void*)&NV,
-                    (void*)&sigma};
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_tasks * GB);
-    cfg.blockDim = dim3(PT);
-    cfg.dynamicSmemBytes = master_persist_smem(max_V, GB);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelExC(&cfg, (const void*)k_master_persist<true>, args);
-    ++*launches;
-    return e;
+    const int most = num_sms / GB;  // plans of one launch: every block resident
+    for (int t0 = 0; t0 < n_tasks; t0 += most) {
+        const MasterTask* part = tasks + t0;
+        void* args[] = {(void*)&none, (void*)&part, (void*)&GB, (void*)&K, (void*)&sigma};
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(std::min(most, n_tasks - t0) * GB);
+        cfg.blockDim = dim3(PT);
+        cfg.dynamicSmemBytes = RING_BYTES;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelExC(&cfg, (const void*)k_master_persist<true>, args);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_cg_record(const MasterDev* st, CGDev* cg, int K, cudaStream_t stream, int* launches) {

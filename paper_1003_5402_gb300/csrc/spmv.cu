@@ -367,7 +367,8 @@ __global__ void __launch_bounds__(256) k_column_dev(const int* __restrict__ col,
     for (int i = threadIdx.x; i < nb; i += blockDim.x) smask[i] = mask[i];
     __syncthreads();
     column_body<G>(col, val, seg + (size_t)b * V, seg + (size_t)(b + 1) * V, V, beam_off[b], smask,
-                   slab + (size_t)(K - 1) * ld, 1, (int)(blockIdx.x * blockDim.x), (int)(gridDim.x * blockDim.x));
+                   slab_column(slab, ld, K - 1), SLAB_STRIDE, (int)(blockIdx.x * blockDim.x),
+                   (int)(gridDim.x * blockDim.x));
 }
 
 // a4 from D by beams, for beam b (b_dev: the beam read from the device's
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(256) k_column_beam(const int* __restrict__ brp
         b = ap_beam[K - 1];
         nb = rows[b] * cols[b];
         base = beam_off[b];
-        out += (size_t)(K - 1) * ld;
+        out = slab_column(out, ld, K - 1);
     }
     for (int i = threadIdx.x; i < nb; i += blockDim.x) smask[i] = W16 ? mask[i] * scale[base + i] : mask[i];
     __syncthreads();
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(256) k_column16_dev(const unsigned short* __re
     for (int i = threadIdx.x; i < nb; i += blockDim.x) smask[i] = mask[i] * scale[base + i];
     __syncthreads();
     column16_body<G, BF>(col, val, seg + (size_t)b * V, seg + (size_t)(b + 1) * V, V, base, smask,
-                         slab + (size_t)(K - 1) * ld, 1, (int)(blockIdx.x * blockDim.x),
+                         slab_column(slab, ld, K - 1), SLAB_STRIDE, (int)(blockIdx.x * blockDim.x),
                          (int)(gridDim.x * blockDim.x));
 }
 
@@ -883,17 +884,17 @@ __global__ void __launch_bounds__(256) k_commit_column(const int* __restrict__ c
             smask[i] = m * scale[base + i];
     }
     __syncthreads();
-    float* out = ca.slab + (size_t)(K - 1) * ca.ld;
+    float* out = slab_column(ca.slab, ca.ld, K - 1);
     const int* seg_lo = ca.seg + (size_t)b * V;
     const int* seg_hi = ca.seg + (size_t)(b + 1) * V;
     if constexpr (G == 0)  // D by beams
         column_beam_body<PREC != DAO_PREC_FP32, PREC == DAO_PREC_BF16>(
-            brp_all + (size_t)b * (V + 1), beam_entry_base(brp_all, V, b), bcol, bval32, bval16, V, smask, out, 1,
+            brp_all + (size_t)b * (V + 1), beam_entry_base(brp_all, V, b), bcol, bval32, bval16, V, smask, out, SLAB_STRIDE,
             (int)(blockIdx.x * blockDim.x), (int)(gridDim.x * blockDim.x));
     else if constexpr (PREC == DAO_PREC_FP32)
-        column_body<G>(col, val, seg_lo, seg_hi, V, base, smask, out, 1, (int)(blockIdx.x * blockDim.x), (int)(gridDim.x * blockDim.x));
+        column_body<G>(col, val, seg_lo, seg_hi, V, base, smask, out, SLAB_STRIDE, (int)(blockIdx.x * blockDim.x), (int)(gridDim.x * blockDim.x));
     else
-        column16_body<G, PREC == DAO_PREC_BF16>(col16, val16, seg_lo, seg_hi, V, base, smask, out, 1, (int)(blockIdx.x * blockDim.x), (int)(gridDim.x * blockDim.x));
+        column16_body<G, PREC == DAO_PREC_BF16>(col16, val16, seg_lo, seg_hi, V, base, smask, out, SLAB_STRIDE, (int)(blockIdx.x * blockDim.x), (int)(gridDim.x * blockDim.x));
 }
 
 // Blocks of a grid-stride kernel that are all resident at once (every block
@@ -1265,7 +1266,7 @@ cudaError_t launch_column_dev(const DevCSR& D, const int* seg, const int* ap_bea
     if (D.n_rows == 0) return cudaSuccess;
     const int grid = num_sms * 8;
     if (column_by_beams(D)) {
-        column_beam_launch(D, 0, 0, 0, ap_beam, K, beam_off, rows, cols, max_nb, mask, slab, 1, ld, cg, grid,
+        column_beam_launch(D, 0, 0, 0, ap_beam, K, beam_off, rows, cols, max_nb, mask, slab, SLAB_STRIDE, ld, cg, grid,
                            stream);
         ++*launches;
         return cudaGetLastError();

@@ -1,0 +1,71 @@
+"""The persistent master solve where its forms change: the tiles of a warp all
+held in shared memory, several ahead or less than two (pool sizes and block
+counts), ragged and single tiles, pools extended by one aperture or by several
+(whose columns come from one pass over their beam's part of D),
+many voxels changing state at once, and D with negative entries (the dose sum
+that needs non-negative terms is then not taken).  The objective at every pool
+size is within the repository's bar (1e-5 relative) of the FP64 oracle's master
+optimum for the same apertures, and bitwise the same in a second run."""
+import numpy as np
+import pytest
+
+import oracle as O
+from _helpers import need_cuda, quantized_case, random_case
+
+pytestmark = pytest.mark.gpu
+
+RTOL_F = 1e-5
+
+
+@pytest.fixture(scope="module")
+def torch():
+    t = need_cuda()
+    from paper_1003_5402_gb300 import build
+    build.build()
+    return t
+
+
+def _pool(case, n, seed):
+    """n different apertures."""
+    rng = np.random.default_rng(seed)
+    seen, out = set(), []
+    while len(out) < n:
+        b = int(rng.integers(case.n_beams))
+        lr = np.sort(rng.integers(0, case.cols[b] + 1, size=(case.rows[b], 2)), axis=1).astype(np.int32)
+        key = (b, lr.tobytes())
+        if key not in seen and np.any(lr[:, 1] > lr[:, 0]):
+            seen.add(key)
+            out.append((b, lr))
+    return out
+
+
+@pytest.mark.parametrize("V,blocks,sizes,negative,prec", [
+    (31, 0, (1, 5), False, "fp32"), (33, 1, (2, 7), False, "fp16"),
+    (700, 0, (3, 4, 12, 13, 40, 41), False, "bf16"), (700, 2, (3, 4, 63, 64), True, "fp32"),
+    (5000, 1, (3, 4, 9, 10, 14, 20, 21, 28, 40, 41, 44, 45, 64), False, "fp32"),
+    (5000, 3, (5, 6, 40, 41), True, "fp16"),
+    (9000, 1, (12, 13, 30, 31), False, "fp16"), (9000, 0, (2, 17, 18, 48), True, "fp32"),
+])
+def test_master_forms_match_the_oracle(torch, V, blocks, sizes, negative, prec):
+    from paper_1003_5402_gb300 import Plan, binding
+    case = random_case(300 + V, V, rows=[5, 4, 6], cols=[7, 9, 5], mean_row=12.0)
+    if negative:
+        rng = np.random.default_rng(V)
+        case.data = np.where(rng.random(len(case.data)) < 0.1, -0.3 * case.data, case.data).astype(np.float32)
+    pool = _pool(case, sizes[-1], 7 * V + blocks)
+    ref_case = case if prec == "fp32" else quantized_case(case, prec)
+    D, vt = O.csr64(ref_case), O.voxel_terms(case)
+    S = np.stack([O.aperture_column(D, ref_case, b, lv) for b, lv in pool], axis=1)
+    got = []
+    for _ in range(2):
+        with Plan(case, master_blocks=blocks, precision={"fp32": binding.DAO_PREC_FP32, "fp16": binding.DAO_PREC_FP16,
+                                                         "bf16": binding.DAO_PREC_BF16}[prec]) as p:
+            K, F = 0, []
+            for k in sizes:
+                F.append(p.import_apertures(pool[K:k]))
+                K = k
+            got.append((F, p.intensities()))
+    assert got[0][0] == got[1][0] and np.array_equal(got[0][1], got[1][1])
+    for k, F in zip(sizes, got[0][0]):
+        ref = O.solve_master(S[:, :k], vt)
+        assert abs(F - ref.F) <= RTOL_F * abs(ref.F), (k, F, ref.F)
