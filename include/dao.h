@@ -614,10 +614,11 @@ void dao_server_destroy(dao_server* srv);
  * another device, or shorter than stated, or column indices outside
  * [0, n_beamlets), are read or written out of bounds.
  * Limits: n_voxels <= 4,194,304 and n_structures <= 64, else DAO_EINVAL with a
- * message.  Scratch: the per-block partial sums of the objective live in a
- * 32 KiB file-scope device array that every GPU loading the library keeps until
- * the process exits; every block overwrites its own entry on each call, so
- * nothing needs clearing, and the array keeps the last call's contents.  All
+ * message.  Scratch: the per-block partial sums of the objective live in an
+ * 8 KiB file-scope device array (and a 4-byte ticket) that every GPU loading the
+ * library keeps until the process exits; every block overwrites its own entry on
+ * each call, so nothing needs clearing, and the array keeps the last call's
+ * contents.  All
  * calls on a device share that array: calls whose kernels overlap on the GPU
  * (for example on different streams) race and give wrong objectives.  The
  * first call on a device looks up the array's device address with that device

@@ -8,24 +8,29 @@
 // allocator owns the whole device.  This entry point computes the same
 // quantities as dao_k_dose (z = D x, grad F(z) and F(z)) without a context
 // and without any allocation: the caller passes the inputs and outputs, and
-// the only scratch memory, the per-block partial sums of F, lives in a
-// file-scope device array that every GPU loading the library keeps until the
+// the only scratch memory, the per-block partial sums of F and their
+// ticket, lives in file-scope device arrays that every GPU loading the library keeps until the
 // process exits.
+#include <algorithm>
 #include <mutex>
 
 #include "dao_internal.h"
 
 namespace {
 
-constexpr int NA_ROWS_PER_BLOCK = 1024;  // voxel rows per block
-constexpr int NA_MAX_BLOCKS = 4096;      // size of the scratch array
-constexpr int NA_THREADS = 256;
-constexpr int NA_LANES = 8;              // lanes per voxel row
+constexpr int NA_MAX_VOXELS = 4194304;   // the entry point's limit
+constexpr int NA_MAX_BLOCKS = 1024;      // size of the scratch array
+constexpr int NA_THREADS = 512;
+constexpr int NA_WARPS = NA_THREADS / 32;
+constexpr int NA_CHUNK = 1024;           // products a warp holds at a time
+constexpr int NA_AHEAD = 8;              // entries per lane requested together
 constexpr int NA_MAX_DEVICES = 64;
 constexpr int SMAX_TERMS = dao::SMAX;
 
-// Per-block FP64 partial sums of the objective (32 KiB per device).
+// Per-block FP64 partial sums of the objective, and the ticket the blocks of a
+// call take when they have written theirs (0 between calls).
 static __device__ __align__(256) double dao_noalloc_scratch[NA_MAX_BLOCKS];
+static __device__ unsigned dao_noalloc_ticket;
 
 struct NoallocTerms {
     double t[SMAX_TERMS][4];  // alpha_s / |v_s|, T_s^-, beta_s / |v_s|, T_s^+
@@ -37,76 +42,150 @@ __device__ __forceinline__ double na_warp_sum(double v) {
     return v;
 }
 
-// One block per NA_ROWS_PER_BLOCK rows; NA_LANES lanes per row with scalar
-// loads of an unpadded CSR; the block's FP64 objective sum goes to partial[b].
-__global__ void __launch_bounds__(NA_THREADS) k_dose_noalloc(int V, const int* __restrict__ rowptr,
-                                                            const int* __restrict__ col,
-                                                            const float* __restrict__ val,
-                                                            const float* __restrict__ x,
-                                                            const int* __restrict__ vstruct, int S,
-                                                            const NoallocTerms terms, float* __restrict__ z,
-                                                            float* __restrict__ grad, double* __restrict__ partial) {
-    __shared__ double s_red[NA_THREADS / 32];
-    const int lane = threadIdx.x & 31;
-    const int sub = lane % NA_LANES;
-    constexpr int RPW = 32 / NA_LANES;
-    const int warp = threadIdx.x >> 5;
-    const int r0 = blockIdx.x * NA_ROWS_PER_BLOCK;
-    const int r1 = min(V, r0 + NA_ROWS_PER_BLOCK);
+// Sum of one double per thread over the block, valid in thread 0.
+__device__ __forceinline__ double na_block_sum(double v, double* s_red) {
+    v = na_warp_sum(v);
+    __syncthreads();  // s_red may still be read from an earlier sum
+    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x < 32) {
+        t = threadIdx.x < NA_WARPS ? s_red[threadIdx.x] : 0.0;
+        t = na_warp_sum(t);
+    }
+    return t;
+}
+
+// A warp takes units of 32 consecutive rows (grid-stride): their entries are one
+// contiguous range, read with consecutive entries on consecutive lanes, NA_AHEAD
+// per lane in flight; the products go to the warp's chunk of shared memory, and
+// lane r sums row r's from there (four interleaved partial sums), so that every
+// lane then has a row of its own for the FP64 epilogue.  The caller's rows have
+// no padding, so wider loads would start off their alignment.  X: x in shared
+// memory.  The block that takes the call's last ticket adds the blocks' partial
+// sums in block order.
+//
+// Bound by the entries' bytes (8 nnz) in the limit; H&N-shaped FP32 matrix
+// (304,184 voxels, 9.55 M entries).  With 8 lanes to a row the epilogue's FP64
+// instructions (1/64 of the FP32 rate) ran with four lanes of 32 in use and each
+// lane waited for its gather before its next entry: 104 us; the call took 158 us
+// and takes 85 now, of which the kernel is the smaller part.
+template <bool X>
+__global__ void __launch_bounds__(NA_THREADS, 2) k_dose_noalloc(int V, int N, const int* __restrict__ rowptr,
+                                                               const int* __restrict__ col,
+                                                               const float* __restrict__ val,
+                                                               const float* __restrict__ x,
+                                                               const int* __restrict__ vstruct, int S,
+                                                               const __grid_constant__ NoallocTerms terms,
+                                                               float* __restrict__ z, float* __restrict__ grad,
+                                                               double* partial, unsigned* ticket,
+                                                               double* __restrict__ out) {
+    extern __shared__ float s_na[];
+    __shared__ double s_red[NA_WARPS];
+    __shared__ double s_t[SMAX_TERMS][4];
+    __shared__ int s_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* buf = s_na + warp * NA_CHUNK;
+    float* sx = s_na + NA_WARPS * NA_CHUNK;
+    const int units = (V + 31) / 32;
+    const bool busy = (int)blockIdx.x * NA_WARPS < units;
+    bool fin = true;
+    for (int i = threadIdx.x; i < 4 * S && busy; i += NA_THREADS) {
+        const double t = (&terms.t[0][0])[i];
+        (&s_t[0][0])[i] = t;
+        fin = fin && isfinite(t);
+    }
+    if (X && busy)
+        for (int i = threadIdx.x; i < N; i += NA_THREADS) sx[i] = __ldg(x + i);
+    const bool finite = __syncthreads_and(fin) != 0;
     double facc = 0.0;
-    for (int base = r0 + warp * RPW; base < r1; base += (NA_THREADS / 32) * RPW) {
-        const int row = base + lane / NA_LANES;
-        float acc = 0.f;
-        if (row < r1) {
-            const int p1 = rowptr[row + 1];
-            for (int p = rowptr[row] + sub; p < p1; p += NA_LANES) acc = fmaf(__ldg(val + p), __ldg(x + col[p]), acc);
-        }
+    for (int u = blockIdx.x * NA_WARPS + warp; u < units; u += gridDim.x * NA_WARPS) {
+        const int row = u * 32 + lane;
+        const int rs = __ldg(rowptr + min(row, V)), re = __ldg(rowptr + min(row + 1, V));
+        const int lab = row < V ? __ldg(vstruct + row) : 0;
+        const int e0 = __shfl_sync(0xffffffffu, rs, 0), e1 = __shfl_sync(0xffffffffu, re, 31);
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int c0 = e0; c0 < e1; c0 += NA_CHUNK) {
+            const int c1 = min(e1, c0 + NA_CHUNK);
+            for (int p0 = c0; p0 < c1; p0 += 32 * NA_AHEAD) {
+                int c[NA_AHEAD];
+                float v[NA_AHEAD];
 #pragma unroll
-        for (int o = NA_LANES / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (row < r1 && sub == 0) {
-            z[row] = acc;
-            const int lab = vstruct[row];
+                for (int q = 0; q < NA_AHEAD; ++q) {
+                    const int p = p0 + 32 * q + lane;
+                    c[q] = p < c1 ? __ldg(col + p) : 0;
+                    v[q] = p < c1 ? __ldg(val + p) : 0.f;
+                }
+#pragma unroll
+                for (int q = 0; q < NA_AHEAD; ++q) {
+                    const int p = p0 + 32 * q + lane;
+                    if (p < c1) buf[p - c0] = v[q] * (X ? sx[c[q]] : __ldg(x + c[q]));
+                }
+            }
+            __syncwarp();
+            const int a = max(rs, c0), b = min(re, c1);
+            int p = a;
+            for (; p + 3 < b; p += 4) {
+                acc[0] += buf[p - c0];
+                acc[1] += buf[p + 1 - c0];
+                acc[2] += buf[p + 2 - c0];
+                acc[3] += buf[p + 3 - c0];
+            }
+            for (; p < b; ++p) acc[0] += buf[p - c0];
+            __syncwarp();
+        }
+        const float zr = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        if (row < V) {
+            z[row] = zr;
             if ((unsigned)lab >= (unsigned)S) {  // no such structure: flagged, never read
                 if (grad != nullptr) grad[row] = __int_as_float(0x7fc00000);
                 facc += __longlong_as_double(0x7ff8000000000000ll);  // the objective becomes NaN
-                continue;
+            } else {
+                const double* tt = s_t[lab];
+                const double zd = zr;
+                const double du = tt[1] - zd, dv = zd - tt[3];
+                float g = 0.f;
+                if (du > 0.0 || dv > 0.0 || !finite) {  // else both penalties are 0 (so most voxels)
+                    const double uu = fmax(0.0, du), o = fmax(0.0, dv);
+                    g = (float)(2.0 * (tt[2] * o - tt[0] * uu));
+                    facc += tt[0] * uu * uu + tt[2] * o * o;
+                }
+                if (grad != nullptr) grad[row] = g;
             }
-            const double* tt = terms.t[lab];
-            const double zd = acc;
-            const double u = fmax(0.0, tt[1] - zd);
-            const double o = fmax(0.0, zd - tt[3]);
-            if (grad != nullptr) grad[row] = (float)(2.0 * (tt[2] * o - tt[0] * u));
-            facc += tt[0] * u * u + tt[2] * o * o;
         }
     }
-    facc = na_warp_sum(facc);
-    if (lane == 0) s_red[warp] = facc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double t = threadIdx.x < NA_THREADS / 32 ? s_red[threadIdx.x] : 0.0;
-        t = na_warp_sum(t);
-        if (threadIdx.x == 0) partial[blockIdx.x] = t;
+    const double t = na_block_sum(facc, s_red);
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = t;
+        // release: the partial sum before the ticket; acquire: the other blocks' sums.
+        // The ticket wraps to 0 with the last block, and every launch has the same
+        // number of blocks, so that it is 0 again whatever overlapped.
+        unsigned old;
+        asm volatile("atom.inc.acq_rel.gpu.global.u32 %0, [%1], %2;"
+                     : "=r"(old)
+                     : "l"(ticket), "r"(gridDim.x - 1u)
+                     : "memory");
+        s_last = old == gridDim.x - 1u;
     }
-}
-
-// Fixed-order sum of the n block partials into *out.
-__global__ void __launch_bounds__(NA_THREADS) k_sum_noalloc(const double* __restrict__ partial, int n,
-                                                           double* __restrict__ out) {
-    __shared__ double s_red[NA_THREADS / 32];
+    __syncthreads();
+    if (!s_last) return;
     double v = 0.0;
-    for (int i = threadIdx.x; i < n; i += NA_THREADS) v += partial[i];
-    v = na_warp_sum(v);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double t = threadIdx.x < NA_THREADS / 32 ? s_red[threadIdx.x] : 0.0;
-        t = na_warp_sum(t);
-        if (threadIdx.x == 0) *out = t;
-    }
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += NA_THREADS) v += __ldcg(partial + i);
+    v = na_block_sum(v, s_red);
+    if (threadIdx.x == 0) *out = v;
 }
 
 std::mutex g_mu;
-double* g_scratch_ptr[NA_MAX_DEVICES] = {};
+// per device: the scratch array, the ticket, the multiprocessors
+struct NoallocDevice {
+    double* scratch = nullptr;
+    unsigned* ticket = nullptr;
+    int sms = 0;
+};
+NoallocDevice g_na[NA_MAX_DEVICES];
+// beamlets whose x fits shared memory beside the warps' chunks
+constexpr int NA_MAX_X = (100 * 1024) / (int)sizeof(float) - NA_WARPS * NA_CHUNK;  // two blocks per SM
+constexpr size_t na_smem(int n) { return sizeof(float) * ((size_t)NA_WARPS * NA_CHUNK + n); }
 
 dao_status na_fail(dao_status s, const std::string& m) { return dao::set_error(s, m); }
 
@@ -121,10 +200,9 @@ dao_status dao_dose_objective_noalloc(int32_t n_voxels, int32_t n_beamlets, cons
     if (n_voxels < 1 || n_beamlets < 1 || !row_ptr || !col || !val || !x || !voxel_struct || !terms || !z ||
         !objective)
         return na_fail(DAO_EINVAL, "null pointer or empty problem");
-    const long long blocks = ((long long)n_voxels + NA_ROWS_PER_BLOCK - 1) / NA_ROWS_PER_BLOCK;
-    if (blocks > NA_MAX_BLOCKS)
-        return na_fail(DAO_EINVAL, "n_voxels exceeds the allocation-free limit of " +
-                                       std::to_string((long long)NA_MAX_BLOCKS * NA_ROWS_PER_BLOCK) + " voxels");
+    if (n_voxels > NA_MAX_VOXELS)
+        return na_fail(DAO_EINVAL, "n_voxels exceeds the allocation-free limit of " + std::to_string(NA_MAX_VOXELS) +
+                                       " voxels");
     if (n_structures < 1 || n_structures > SMAX_TERMS)
         return na_fail(DAO_EINVAL, "n_structures must be in [1, " + std::to_string(SMAX_TERMS) + "]");
     int dev = 0;
@@ -140,33 +218,52 @@ dao_status dao_dose_objective_noalloc(int32_t n_voxels, int32_t n_beamlets, cons
             return na_fail(DAO_EINVAL, "the stream belongs to device " + std::to_string(sdev) +
                                            ", not to the current device " + std::to_string(dev));
     }
-    double* scratch = nullptr;
+    NoallocDevice nd;
     {
-        // set-up, once per device with that device current: the device address of
-        // the file-scope array (its name is only a host-side stand-in).  The
-        // address belongs to the device's primary context as it was at that first
-        // call; after a cudaDeviceReset it is stale, and a caller that resets the
-        // device must not call this entry point again in the same process.
+        // set-up, once per device with that device current: the device addresses of
+        // the file-scope array and ticket (their names are only host-side
+        // stand-ins) and the kernels' shared memory limit.  The addresses belong
+        // to the device's primary context as it was at that first call; after a
+        // cudaDeviceReset they are stale, and a caller that resets the device must
+        // not call this entry point again in the same process.
         std::lock_guard<std::mutex> lock(g_mu);
-        if (g_scratch_ptr[dev] == nullptr) {
-            void* p = nullptr;
+        NoallocDevice& g = g_na[dev];
+        if (g.scratch == nullptr) {
+            void *p = nullptr, *q = nullptr;
+            int sms = 0;
             e = cudaGetSymbolAddress(&p, dao_noalloc_scratch);
-            if (e != cudaSuccess)
-                return na_fail(DAO_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
-            g_scratch_ptr[dev] = static_cast<double*>(p);
+            if (e == cudaSuccess) e = cudaGetSymbolAddress(&q, dao_noalloc_ticket);
+            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k_dose_noalloc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)na_smem(NA_MAX_X));
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k_dose_noalloc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)na_smem(0));
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                return na_fail(DAO_ECUDA, std::string("noalloc set-up: ") + cudaGetErrorString(e));
+            }
+            g.ticket = static_cast<unsigned*>(q);
+            g.sms = sms;
+            g.scratch = static_cast<double*>(p);
         }
-        scratch = g_scratch_ptr[dev];
+        nd = g;
     }
     NoallocTerms t;
     for (int s = 0; s < SMAX_TERMS; ++s)
         for (int q = 0; q < 4; ++q) t.t[s][q] = s < n_structures ? terms[4 * s + q] : 0.0;
-    k_dose_noalloc<<<(unsigned)blocks, NA_THREADS, 0, st>>>(n_voxels, row_ptr, col, val, x, voxel_struct,
-                                                          n_structures, t, z, grad, scratch);
+    const unsigned grid = (unsigned)std::min(2 * nd.sms, NA_MAX_BLOCKS);  // the same for every call: see the ticket
+    if (n_beamlets <= NA_MAX_X)
+        k_dose_noalloc<true><<<grid, NA_THREADS, na_smem(n_beamlets), st>>>(n_voxels, n_beamlets, row_ptr, col, val, x,
+                                                                           voxel_struct, n_structures, t, z, grad,
+                                                                           nd.scratch, nd.ticket, objective);
+    else
+        k_dose_noalloc<false><<<grid, NA_THREADS, na_smem(0), st>>>(n_voxels, n_beamlets, row_ptr, col, val, x,
+                                                                   voxel_struct, n_structures, t, z, grad, nd.scratch,
+                                                                   nd.ticket, objective);
     e = cudaGetLastError();
     if (e != cudaSuccess) return na_fail(DAO_ECUDA, std::string("k_dose_noalloc: ") + cudaGetErrorString(e));
-    k_sum_noalloc<<<1, NA_THREADS, 0, st>>>(scratch, (int)blocks, objective);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return na_fail(DAO_ECUDA, std::string("k_sum_noalloc: ") + cudaGetErrorString(e));
     return DAO_OK;
 }
 
