@@ -118,7 +118,6 @@ struct dao_ctx {
     bool solve_tried = false;
     double* F_part = nullptr;
     int F_blocks = 0;
-    double* F_dev = nullptr;
 
     // pinned staging
     unsigned char* pinned = nullptr;
@@ -683,7 +682,8 @@ dao_status alloc_state(dao_ctx* c) {
     DAO_TRY(c->dalloc(&c->mb.F_part, (size_t)master_grid_max(c->num_sms)));
     c->F_blocks = std::max(dose_grid(c->V, c->num_sms), dose_merge_f_slots(c->D));
     DAO_TRY(c->dalloc(&c->F_part, c->F_blocks));
-    DAO_TRY(c->dalloc(&c->F_dev, 1));
+    DAO_TRY(c->dalloc(&c->D.f_ticket, 1));
+    DAO_CU(cudaMemsetAsync(c->D.f_ticket, 0, sizeof(unsigned), c->stream));
     DAO_CU(cudaMemsetAsync(c->mb.st, 0, sizeof(MasterDev), c->stream));
     DAO_CU(cudaMemsetAsync(c->ap_lr, 0, (size_t)c->K_cap * 2 * c->max_rows * sizeof(int), c->stream));
     c->off_small = 0;
@@ -1526,15 +1526,28 @@ dao_status dao_sizes(const dao_ctx* c, int32_t* V, int32_t* N, int32_t* B, int32
 
 dao_status dao_price(dao_ctx* c, int32_t* beam, int32_t* leaf_lr, double* rc) {
     DAO_TRY(check_ctx(c));
+    // D^T with the MLC-row search in its blocks (an MLC constraint: the beams
+    // priced by their own kernel), then the beam decision, which writes the
+    // outcome to the page-locked block itself
+    const bool mlc = c->opt.mlc_constraint != DAO_MLC_CONSECUTIVE;
+    const RowTicket rt{c->binfo, c->beam_row0_d, c->cols_d, c->row_info, mlc ? nullptr : c->row_cnt,
+                       c->row_v, c->row_lr, nullptr};
+    PriceDev* pd = reinterpret_cast<PriceDev*>(c->pinned + c->off_small + 16);
+    int* lr = reinterpret_cast<int*>(c->pinned + c->off_rows);
     c->prof_begin(DAO_KC_DT);
-    DAO_CU(launch_dt(c->Dt, c->pi, c->w, nullptr, c->stream, &c->launches_i));
+    DAO_CU(launch_dt_rows(c->Dt, c->pi, c->w, rt, c->stream, &c->launches_i));
     c->prof_end();
-    double r = 0.0;
-    dao_status st = price_on_w(c, c->w, beam, leaf_lr, &r, nullptr, nullptr);
+    c->prof_begin(DAO_KC_PRICE);
+    if (mlc) DAO_CU(price_rows_any(c, c->w, nullptr, c->stream, &c->launches_i));
+    DAO_CU(launch_price_beams(c->row_v, c->beam_row0_d, c->B, pd, nullptr, c->stream, &c->launches_i, c->row_lr,
+                              reinterpret_cast<int2*>(lr)));
+    c->prof_end();
+    DAO_TRY(sync(c));
     c->count_launches();
-    if (st != DAO_OK) return st;
-    if (rc) *rc = r;
-    return r < -c->tau ? DAO_OK : DAO_OPTIMAL;
+    if (beam) *beam = pd->beam;
+    if (leaf_lr) std::memcpy(leaf_lr, lr, sizeof(int) * 2 * (size_t)c->rows[pd->beam]);
+    if (rc) *rc = pd->rc;
+    return pd->rc < -c->tau ? DAO_OK : DAO_OPTIMAL;
 }
 
 dao_status dao_import_apertures(dao_ctx* c, int32_t n, const int32_t* beams, const int32_t* leaf_lr,
@@ -1622,12 +1635,11 @@ dao_status dao_dose(dao_ctx* c, float* dose, double* objective) {
     DAO_TRY(check_ctx(c));
     DAO_CU(launch_fluence(c->ap_beam, c->ap_lr, 2 * c->max_rows, c->mb.st->y, c->K, c->binfo, c->N, c->x, c->stream,
                           &c->launches_i));
+    double* f = reinterpret_cast<double*>(c->pinned + c->off_small + 8);  // the kernel writes F there itself
     c->prof_begin(DAO_KC_DOSE);
-    DAO_CU(launch_dose(c->D, c->x, c->vstruct, c->tf, c->ts, c->S, c->dose, nullptr, c->F_part, c->F_blocks, c->F_dev,
+    DAO_CU(launch_dose(c->D, c->x, c->vstruct, c->tf, c->ts, c->S, c->dose, nullptr, c->F_part, c->F_blocks, f,
                        c->num_sms, c->stream, &c->launches_i));
     c->prof_end();
-    double* f = reinterpret_cast<double*>(c->pinned + c->off_small + 8);
-    DAO_CU(cudaMemcpyAsync(f, c->F_dev, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     if (dose) DAO_CU(cudaMemcpyAsync(dose, c->dose, sizeof(float) * c->V, cudaMemcpyDeviceToHost, c->stream));
     DAO_TRY(sync(c));
     if (objective) *objective = *f;
@@ -1683,9 +1695,8 @@ dao_status dao_fmo(dao_ctx* c, int32_t max_iters, double tol, double* x_out, dou
     int* n = &c->launches_i;
     // F, z and pi of x: the a1 kernel with its epilogue; g = D^T pi: the a2 kernel
     auto evaluate = [&](const float* x32, float* z, float* pi) -> dao_status {
-        DAO_CU(launch_dose(c->D, x32, c->vstruct, c->tf, c->ts, c->S, z, pi, c->F_part, c->F_blocks, c->F_dev,
+        DAO_CU(launch_dose(c->D, x32, c->vstruct, c->tf, c->ts, c->S, z, pi, c->F_part, c->F_blocks, hF,
                            c->num_sms, s, n));
-        DAO_CU(cudaMemcpyAsync(hF, c->F_dev, sizeof(double), cudaMemcpyDeviceToHost, s));
         return DAO_OK;
     };
     auto read_scalars = [&]() -> dao_status {
@@ -1764,18 +1775,13 @@ dao_status dao_fmo(dao_ctx* c, int32_t max_iters, double tol, double* x_out, dou
 dao_status dao_k_dose(dao_ctx* c, const float* x, float* z, float* grad, double* objective) {
     DAO_TRY(check_ctx(c));
     if (!x || !z) return fail(DAO_EINVAL, "null vector");
+    double* f = reinterpret_cast<double*>(c->pinned + c->off_small + 8);  // the kernel writes F there itself
     c->prof_begin(DAO_KC_DOSE);
     DAO_CU(launch_dose(c->D, x, c->vstruct, c->tf, c->ts, c->S, z, grad, objective ? c->F_part : nullptr, c->F_blocks,
-                       c->F_dev, c->num_sms, c->stream, &c->launches_i));
+                       f, c->num_sms, c->stream, &c->launches_i));
     c->prof_end();
-    if (objective) {
-        double* f = reinterpret_cast<double*>(c->pinned + c->off_small + 8);
-        DAO_CU(cudaMemcpyAsync(f, c->F_dev, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        DAO_TRY(sync(c));
-        *objective = *f;
-    } else {
-        DAO_TRY(sync(c));
-    }
+    DAO_TRY(sync(c));
+    if (objective) *objective = *f;
     c->count_launches();
     return DAO_OK;
 }

@@ -67,6 +67,7 @@ struct DevCSR {
     int* rowptr = nullptr;   // n_rows + 1; multiples of 4 (FP32) or 8 (16-bit values)
     int* col = nullptr;      // FP32 layout, and the voxel indices of a 16-bit D^T
     float* val = nullptr;    // FP32 values
+    unsigned* f_ticket = nullptr;     // D: ticket of the dose kernel's objective sum (0 between launches)
     unsigned short* col16 = nullptr;  // 16-bit layout of D: beamlet indices
     unsigned short* val16 = nullptr;  // 16-bit values D_ij / s_i (FP16 or BF16 bits)
     const float* scale = nullptr;     // 16-bit layout: per-beamlet scale s_i (length n_beamlets)
@@ -197,7 +198,8 @@ struct CGDev {
 
 // ---- kernel launchers (all on `stream`; return the launch error) ----------
 
-// a1: z = D x, optional grad F(z), FP64 F partials (one per block) reduced into *F_out.
+// a1: z = D x, optional grad F(z), FP64 F partials (one per block) reduced into *F_out
+// (device or page-locked host memory).
 cudaError_t launch_dose(const DevCSR& D, const float* x, const uint8_t* vstruct,
                         const StructTermsF* tf, const StructTermsS* ts, int S,
                         float* z, float* grad, double* F_part, int F_blocks, double* F_out,
@@ -248,9 +250,11 @@ cudaError_t launch_price_commit(const double* row_v, const int* beam_row0, int n
                                 const int2* row_lr, const int* rows, const int* cols, double tau, int K, int lr_stride,
                                 int* ap_beam, int* ap_lr, float* mask, CGDev* cg, cudaStream_t stream, int* launches);
 
-// Only the per-beam sums of row_v and their argmin (k_price_beams).
+// Only the per-beam sums of row_v and their argmin (k_price_beams), with the best
+// beam's rows of row_lr into leaves when that is given.
 cudaError_t launch_price_beams(const double* row_v, const int* beam_row0, int n_beams, PriceDev* out,
-                               const int* skip, cudaStream_t stream, int* launches);
+                               const int* skip, cudaStream_t stream, int* launches, const int2* row_lr = nullptr,
+                               int2* leaves = nullptr);
 // a3 under an MLC constraint (mlc.cu): one block per beam writes row_v (the
 // beam's value at its first row, 0 at the others) and row_lr; smem bytes from
 // mlc_smem_bytes for the largest beam, after mlc_configure with that size.
@@ -290,7 +294,8 @@ dao_status pencil_check(const dao_pencil_beam* pb);
 cudaError_t pencil_generate(const dao_pencil_beam* pb, int device, cudaStream_t s, int64_t** rp, int** col,
                             float** val, int64_t* nnz);
 
-// The device-driven round (one graph for every round of a solve):
+// D^T with the MLC-row search fused (launch_dt_rows), and the device-driven round
+// (one graph for every round of a solve):
 //  - D^T with the MLC-row search fused: the block that completes the last
 //    beamlet of an MLC row (a per-row ticket) runs that row's search; block 0
 //    snapshots cg->K and cg->stop into rs_K and rs_stop;
@@ -307,7 +312,7 @@ struct RowTicket {
     int* row_cnt;           // per MLC row: beamlets done this round (the row's last block resets it)
     double* row_v;
     int2* row_lr;
-    CGDev* cg;
+    CGDev* cg;              // the round's snapshot and stop flag; nullptr outside a device-driven round
 };
 cudaError_t launch_dt_rows(const DevCSR& Dt, const float* pi, float* w, const RowTicket& rt, cudaStream_t stream,
                            int* launches);

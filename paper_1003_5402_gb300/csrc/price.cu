@@ -19,16 +19,17 @@ __global__ void __launch_bounds__(256) k_price_rows(const float* __restrict__ w,
 }
 
 // One block: thread b sums beam b's rows in row order; thread 0 takes the argmin.
+// leaves (nullable): the best beam's leaf positions.  out and leaves may be
+// page-locked host memory, which saves the copies after the kernel.
 __global__ void __launch_bounds__(256) k_price_beams(const double* __restrict__ row_v,
                                                      const int* __restrict__ beam_row0, int n_beams,
-                                                     PriceDev* __restrict__ out, const int* __restrict__ skip) {
+                                                     PriceDev* __restrict__ out, const int2* __restrict__ row_lr,
+                                                     int2* __restrict__ leaves, const int* __restrict__ skip) {
     extern __shared__ double s_sum[];
+    __shared__ int s_best;
     if (skip != nullptr && *skip) return;
-    for (int b = threadIdx.x; b < n_beams; b += blockDim.x) {
-        double t = 0.0;
-        for (int r = beam_row0[b]; r < beam_row0[b + 1]; ++r) t = t + row_v[r];
-        s_sum[b] = t;
-    }
+    for (int b = threadIdx.x; b < n_beams; b += blockDim.x)
+        s_sum[b] = pricing::beam_sum(row_v, beam_row0[b], beam_row0[b + 1]);
     __syncthreads();
     if (threadIdx.x == 0) {
         int best = 0;
@@ -36,7 +37,12 @@ __global__ void __launch_bounds__(256) k_price_beams(const double* __restrict__ 
             if (s_sum[b] < s_sum[best]) best = b;
         out->beam = best;
         out->rc = n_beams > 0 ? s_sum[best] : 0.0;
+        s_best = best;
     }
+    if (leaves == nullptr) return;
+    __syncthreads();
+    const int r0 = beam_row0[s_best], n = beam_row0[s_best + 1] - r0;
+    for (int r = threadIdx.x; r < n; r += blockDim.x) leaves[r] = row_lr[r0 + r];
 }
 
 // The beam sums and their argmin (as k_price_beams) in one block with the
@@ -111,9 +117,9 @@ cudaError_t launch_price_commit(const double* row_v, const int* beam_row0, int n
 }
 
 cudaError_t launch_price_beams(const double* row_v, const int* beam_row0, int n_beams, PriceDev* out,
-                               const int* skip, cudaStream_t stream, int* launches) {
-    k_price_beams<<<1, 256, (size_t)(n_beams > 0 ? n_beams : 1) * sizeof(double), stream>>>(row_v, beam_row0,
-                                                                                           n_beams, out, skip);
+                               const int* skip, cudaStream_t stream, int* launches, const int2* row_lr, int2* leaves) {
+    k_price_beams<<<1, 256, (size_t)(n_beams > 0 ? n_beams : 1) * sizeof(double), stream>>>(
+        row_v, beam_row0, n_beams, out, row_lr, leaves, skip);
     ++*launches;
     return cudaGetLastError();
 }
@@ -131,10 +137,7 @@ cudaError_t launch_price(const float* w, const int4* row_info, int n_rows, const
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    k_price_beams<<<1, 256, (size_t)(n_beams > 0 ? n_beams : 1) * sizeof(double), stream>>>(row_v, beam_row0,
-                                                                                           n_beams, out, skip);
-    ++*launches;
-    return cudaGetLastError();
+    return launch_price_beams(row_v, beam_row0, n_beams, out, skip, stream, launches);
 }
 
 }  // namespace dao

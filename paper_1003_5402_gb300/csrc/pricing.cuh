@@ -89,6 +89,23 @@ __device__ __forceinline__ void row_best(const float* __restrict__ w, int4 ri, i
     }
 }
 
+// Sum of rows [r0, r1) of row_v in row order, 16 rows requested before the first
+// add (a plain loop waits for L2 at every add).  Not for decide below: there the
+// registers would cost the fused column kernel's occupancy (a plan of 50
+// apertures, H&N-shaped: 7.31 against 6.71 ms).
+__device__ __forceinline__ double beam_sum(const double* __restrict__ row_v, int r0, int r1) {
+    double t = 0.0;
+    for (int r = r0; r < r1; r += 16) {
+        double v[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = r + q < r1 ? __ldcg(row_v + r + q) : 0.0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+            if (r + q < r1) t = t + v[q];
+    }
+    return t;
+}
+
 enum { OUTCOME_NEW = 0, OUTCOME_OPTIMAL = 1, OUTCOME_DUPLICATE = 2 };
 
 // Whole block (every thread calls it): beam sums into s_sum (n_beams doubles

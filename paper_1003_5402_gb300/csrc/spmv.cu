@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(UNIT_THREADS, 2) k_dose_units(
     const int* __restrict__ rowptr, const uint4* __restrict__ colg, const uint4* __restrict__ valg, int V,
     const float* __restrict__ x, const float* __restrict__ scale, int N, const uint8_t* __restrict__ vstruct,
     const StructTermsS* __restrict__ ts, int S, float* __restrict__ z, float* __restrict__ grad,
-    double* __restrict__ F_part, int part_cap) {
+    double* F_part, int part_cap, unsigned* ticket, double* F_out) {
     constexpr int EPG = L16 ? 8 : 4;  // entries per group (one 16-byte load of columns and of values)
     constexpr int UB = 4;             // groups per lane in flight
     constexpr int NW = UNIT_THREADS / 32;
@@ -619,8 +619,27 @@ __global__ void __launch_bounds__(UNIT_THREADS, 2) k_dose_units(
         lab = lab_n;
     }
     if (F_part != nullptr) {
+        // the blocks' sums added in block order by the last block to finish
+        // (256 threads, each every 256th), instead of by a launch of their own
+        __shared__ int s_last;
         const double sres = block_sum_mixed<UNIT_THREADS>(facc, s_red);
-        if (threadIdx.x == 0) F_part[blockIdx.x] = sres;
+        if (threadIdx.x == 0) {
+            F_part[blockIdx.x] = sres;
+            s_last = F_out != nullptr && atom_add_acq_rel_gpu(ticket, 1u) == gridDim.x - 1;
+            if (s_last) *ticket = 0;  // every block has taken its ticket
+        }
+        __syncthreads();
+        if (!s_last) return;
+        double t = 0.0;
+        if (threadIdx.x < 256)
+            for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) t += __ldcg(F_part + i);
+        t = warp_sum_f64(t);
+        if (lane == 0) s_red[wib] = t;
+        __syncthreads();
+        if (wib == 0) {
+            t = warp_sum_f64(lane < 8 ? s_red[lane] : 0.0);
+            if (lane == 0) *F_out = t;
+        }
     }
 }
 
@@ -938,7 +957,8 @@ size_t units_smem(int N, int part_cap) {
 
 template <bool L16, bool BF>
 cudaError_t dose_units(const DevCSR& D, const float* x, const uint8_t* vstruct, const StructTermsS* ts, int S,
-                       float* z, float* grad, double* F_part, int& grid, int num_sms, cudaStream_t stream) {
+                       float* z, float* grad, double* F_part, double* F_out, int& grid, int num_sms,
+                       cudaStream_t stream) {
     const size_t smem = units_smem(D.n_cols, D.unit_groups_max);
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dose_units<L16, BF>, UNIT_THREADS, smem) !=
@@ -952,7 +972,7 @@ cudaError_t dose_units(const DevCSR& D, const float* x, const uint8_t* vstruct, 
     const void* valp = L16 ? static_cast<const void*>(D.val16) : static_cast<const void*>(D.val);
     k_dose_units<L16, BF><<<grid, UNIT_THREADS, smem, stream>>>(
         D.rowptr, static_cast<const uint4*>(colp), static_cast<const uint4*>(valp), D.n_rows, x, D.scale, D.n_cols,
-        vstruct, ts, S, z, grad, F_part, D.unit_groups_max);
+        vstruct, ts, S, z, grad, F_part, D.unit_groups_max, D.f_ticket, F_out);
     return cudaGetLastError();
 }
 
@@ -1141,11 +1161,11 @@ cudaError_t launch_dose(const DevCSR& D, const float* x, const uint8_t* vstruct,
         return cudaGetLastError();
     }
     if (units && D.prec == DAO_PREC_FP32)
-        e = dose_units<false, false>(D, x, vstruct, ts, S, z, grad, F_part, grid, num_sms, stream);
+        e = dose_units<false, false>(D, x, vstruct, ts, S, z, grad, F_part, F_out, grid, num_sms, stream);
     else if (units && D.prec == DAO_PREC_FP16)
-        e = dose_units<true, false>(D, x, vstruct, ts, S, z, grad, F_part, grid, num_sms, stream);
+        e = dose_units<true, false>(D, x, vstruct, ts, S, z, grad, F_part, F_out, grid, num_sms, stream);
     else if (units)
-        e = dose_units<true, true>(D, x, vstruct, ts, S, z, grad, F_part, grid, num_sms, stream);
+        e = dose_units<true, true>(D, x, vstruct, ts, S, z, grad, F_part, F_out, grid, num_sms, stream);
     else if (D.prec == DAO_PREC_BF16)
         e = dose16_any<true>(g, D, x, vstruct, ts, S, z, grad, F_part, grid, num_sms, stream);
     else if (D.prec == DAO_PREC_FP16)
@@ -1159,7 +1179,7 @@ cudaError_t launch_dose(const DevCSR& D, const float* x, const uint8_t* vstruct,
     else
         e = dose_g<32>(D, x, vstruct, ts, S, z, grad, F_part, grid, num_sms, stream);
     ++*launches;
-    if (e != cudaSuccess || F_part == nullptr || F_out == nullptr) return e;
+    if (e != cudaSuccess || F_part == nullptr || F_out == nullptr || units) return e;  // (units: summed in the kernel)
     k_sum_f64<<<1, 256, 0, stream>>>(F_part, grid, F_out);
     ++*launches;
     return cudaGetLastError();
@@ -1207,8 +1227,8 @@ cudaError_t launch_dt(const DevCSR& Dt, const float* pi, float* w, const int* sk
 
 cudaError_t launch_dt_rows(const DevCSR& Dt, const float* pi, float* w, const RowTicket& rt, cudaStream_t stream,
                            int* launches) {
-    if (rt.cg == nullptr) return cudaErrorInvalidValue;  // row_cnt null: the snapshot without the row search
-    return dt_dispatch(Dt, pi, w, &rt.cg->stop, rt, stream, launches);
+    // row_cnt null: the snapshot without the row search
+    return dt_dispatch(Dt, pi, w, rt.cg ? &rt.cg->stop : nullptr, rt, stream, launches);
 }
 
 // The aperture column runs on D by beams when the launch shape is 0 (the
