@@ -871,6 +871,50 @@ dao_status append_aperture(dao_ctx* c, int beam, const int32_t* lr) {
     return DAO_OK;
 }
 
+// The same for n apertures (leaf_lr: 2 * max_rows each): the table entries first,
+// then the columns, several apertures of a beam per launch.
+dao_status append_apertures(dao_ctx* c, int n, const int32_t* beams, const int32_t* leaf_lr) {
+    const int stride = 2 * c->max_rows, K0 = c->K;
+    if (n < 2 || !columns_available(c->D, c->max_nb)) {  // one column per launch
+        for (int i = 0; i < n; ++i) {
+            DAO_TRY(append_aperture(c, beams[i], leaf_lr + (size_t)i * stride));
+            DAO_TRY(sync(c));  // the column's mask is staged in one pinned buffer, refilled by the next aperture
+        }
+        return DAO_OK;
+    }
+    c->ap_beam_h.insert(c->ap_beam_h.end(), beams, beams + n);
+    c->ap_lr_h.resize((size_t)(K0 + n) * stride, 0);
+    std::vector<ColumnList> list(c->B, ColumnList{});
+    for (int i = 0; i < n; ++i) {
+        const int32_t* lr = leaf_lr + (size_t)i * stride;
+        for (int r = 0; r < c->rows[beams[i]]; ++r) {
+            const bool open = lr[2 * r] < lr[2 * r + 1];
+            c->ap_lr_h[(size_t)(K0 + i) * stride + 2 * r] = open ? lr[2 * r] : 0;
+            c->ap_lr_h[(size_t)(K0 + i) * stride + 2 * r + 1] = open ? lr[2 * r + 1] : 0;
+        }
+    }
+    DAO_CU(cudaMemcpyAsync(c->ap_beam + K0, &c->ap_beam_h[K0], sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
+    DAO_CU(cudaMemcpyAsync(c->ap_lr + (size_t)K0 * stride, &c->ap_lr_h[(size_t)K0 * stride],
+                           sizeof(int) * (size_t)n * stride, cudaMemcpyHostToDevice, c->stream));
+    c->prof_begin(DAO_KC_COLUMN);
+    auto flush = [&](int b) -> cudaError_t {
+        const cudaError_t e = launch_columns(c->D, b, c->beam_off[b], c->rows[b], c->cols[b], list[b], c->ap_lr,
+                                             stride, c->slab, c->ld, c->num_sms, c->stream, &c->launches_i);
+        list[b].n = 0;
+        return e;
+    };
+    for (int i = 0; i < n; ++i) {
+        ColumnList& l = list[beams[i]];
+        l.k[l.n++] = K0 + i;
+        if (l.n == COLUMNS_MAX) DAO_CU(flush(beams[i]));
+    }
+    for (int b = 0; b < c->B; ++b)
+        if (list[b].n > 0) DAO_CU(flush(b));
+    c->prof_end();
+    c->K += n;
+    return DAO_OK;
+}
+
 dao_status add_aperture(dao_ctx* c, int beam, const int32_t* lr, double* F) {
     if (c->K >= c->K_cap) return fail(DAO_ESTATE, "aperture pool is full (k_max)");
     DAO_TRY(append_aperture(c, beam, lr));
@@ -1564,10 +1608,7 @@ dao_status dao_import_apertures(dao_ctx* c, int32_t n, const int32_t* beams, con
             return fail(DAO_EINVAL, "starting intensities must be finite and >= 0");
     }
     const int K0 = c->K;
-    for (int i = 0; i < n; ++i) {
-        DAO_TRY(append_aperture(c, beams[i], leaf_lr + (size_t)i * stride));
-        DAO_TRY(sync(c));  // the column's mask is staged in one pinned buffer, refilled by the next aperture
-    }
+    DAO_TRY(append_apertures(c, n, beams, leaf_lr));
     if (n > 0) {
         // the master starts from y_start on the imported apertures (the last at 0,
         // as for every added aperture) and from the current optimum on the rest

@@ -397,6 +397,69 @@ __global__ void __launch_bounds__(256) k_column_beam(const int* __restrict__ brp
                               smask, out, stride, (int)(blockIdx.x * blockDim.x), (int)(gridDim.x * blockDim.x));
 }
 
+// a4 for several apertures of one beam: one pass over the beam's part of D by
+// beams, a bit per aperture and beamlet in shared memory; each column's sum takes
+// the open entries in order, the arithmetic of column_beam_body (a closed
+// entry's product is 0 there).  An imported pool of 40 apertures on the
+// H&N-shaped matrix took 40 launches of 8.8 us with a mask upload and a
+// synchronisation each.
+template <bool W16, bool BF>
+__global__ void __launch_bounds__(256) k_columns_beam(const int* __restrict__ brp_all,
+                                                      const unsigned short* __restrict__ bcol,
+                                                      const float* __restrict__ bval32,
+                                                      const unsigned short* __restrict__ bval16, int V, int b,
+                                                      int base, int rows, int cols,
+                                                      const __grid_constant__ ColumnList list,
+                                                      const int* __restrict__ ap_lr, int lr_stride,
+                                                      const float* __restrict__ scale, float* __restrict__ slab,
+                                                      int ld) {
+    extern __shared__ float2 s_open[];  // per beamlet: the scale (1 for FP32 values), the apertures' bits
+    const int nb = rows * cols;
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+        const int r = i / cols, c = i % cols;
+        unsigned m = 0u;
+        for (int q = 0; q < list.n; ++q) {
+            const int* lr = ap_lr + (size_t)list.k[q] * lr_stride + 2 * r;
+            m |= (c >= lr[0] && c < lr[1] ? 1u : 0u) << q;
+        }
+        s_open[i] = make_float2(W16 ? scale[base + i] : 1.f, __uint_as_float(m));
+    }
+    __syncthreads();
+    const int* brp = brp_all + (size_t)b * (V + 1);
+    const int e_base = beam_entry_base(brp_all, V, b);
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < V; j += gridDim.x * blockDim.x) {
+        const int p0 = __ldg(brp + j) + e_base, p1 = __ldg(brp + j + 1) + e_base;
+        float acc[COLUMNS_MAX];
+#pragma unroll
+        for (int q = 0; q < COLUMNS_MAX; ++q) acc[q] = 0.f;
+        for (int p = p0; p < p1; p += 4) {
+            unsigned short c[4];
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const bool in = p + e < p1;
+                c[e] = in ? __ldg(bcol + p + e) : (unsigned short)0;
+                if constexpr (W16)
+                    v[e] = in ? unpack1<BF>(__ldg(bval16 + p + e)) : 0.f;
+                else
+                    v[e] = in ? __ldg(bval32 + p + e) : 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (p + e < p1) {
+                    const float2 o = s_open[c[e]];
+                    const unsigned m = __float_as_uint(o.y);
+#pragma unroll
+                    for (int q = 0; q < COLUMNS_MAX; ++q)
+                        if ((m >> q) & 1u) acc[q] = fmaf(v[e], o.x, acc[q]);
+                }
+        }
+#pragma unroll
+        for (int q = 0; q < COLUMNS_MAX; ++q)
+            if (q < list.n) slab_column(slab, ld, list.k[q])[(size_t)SLAB_STRIDE * j] = acc[q];
+    }
+}
+
 // ---- Eq. 7 ------------------------------------------------------------------
 __global__ void k_fluence(const int* __restrict__ ap_beam, const int* __restrict__ ap_lr, int lr_stride,
                           const double* __restrict__ y, int K, const int4* __restrict__ binfo, int N,
@@ -1276,6 +1339,33 @@ cudaError_t launch_column(const DevCSR& D, const int* seg, int b, int base, int 
         case 16: column_launch<16>(D, seg_lo, seg_hi, base, nb, mask, out, stride, grid, stream); break;
         default: column_launch<8>(D, seg_lo, seg_hi, base, nb, mask, out, stride, grid, stream); break;
     }
+    ++*launches;
+    return cudaGetLastError();
+}
+
+bool columns_available(const DevCSR& D, int max_nb) {
+    return column_by_beams(D) && (size_t)max_nb * sizeof(float2) <= 48 * 1024;
+}
+
+cudaError_t launch_columns(const DevCSR& D, int b, int base, int rows, int cols, const ColumnList& list,
+                           const int* ap_lr, int lr_stride, float* slab, int ld, int num_sms, cudaStream_t stream,
+                           int* launches) {
+    if (!columns_available(D, rows * cols)) return cudaErrorNotSupported;
+    if (D.n_rows == 0 || list.n == 0) return cudaSuccess;
+    const size_t sm = (size_t)rows * cols * sizeof(float2);
+    const int grid = std::min(num_sms * 8, (D.n_rows + 255) / 256);
+    if (D.prec == DAO_PREC_FP16)
+        k_columns_beam<true, false><<<grid, 256, sm, stream>>>(D.beam_rowptr, D.beam_col, nullptr, D.beam_val16,
+                                                                D.n_rows, b, base, rows, cols, list, ap_lr, lr_stride,
+                                                                D.scale, slab, ld);
+    else if (D.prec == DAO_PREC_BF16)
+        k_columns_beam<true, true><<<grid, 256, sm, stream>>>(D.beam_rowptr, D.beam_col, nullptr, D.beam_val16,
+                                                               D.n_rows, b, base, rows, cols, list, ap_lr, lr_stride,
+                                                               D.scale, slab, ld);
+    else
+        k_columns_beam<false, false><<<grid, 256, sm, stream>>>(D.beam_rowptr, D.beam_col, D.beam_val32, nullptr,
+                                                                 D.n_rows, b, base, rows, cols, list, ap_lr,
+                                                                 lr_stride, D.scale, slab, ld);
     ++*launches;
     return cudaGetLastError();
 }
