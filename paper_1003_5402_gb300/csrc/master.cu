@@ -565,7 +565,9 @@ __device__ __forceinline__ void master_reduce_words(const float* __restrict__ H_
     const int E = K * (K + 1) / 2;
     const int lane = threadIdx.x & 31;
     const int n_out = last_only ? K + 2 : E + 2 * K + 1;
-    for (int o_ = (bid * (int)blockDim.x + (int)threadIdx.x) >> 5; o_ < n_out; o_ += (G * (int)blockDim.x) >> 5) {
+    // consecutive outputs on different blocks: the FP64 sums (g, F) are consecutive,
+    // and an SM's FP64 pipe is slow
+    for (int o_ = bid + G * ((int)threadIdx.x >> 5); o_ < n_out; o_ += G * ((int)blockDim.x >> 5)) {
         const int o = !last_only ? o_ : o_ < K ? E - K + o_ : o_ == K ? E + K - 1 : E + 2 * K - 1;
         if (o < E) {  // the factorisation is FP32: so is this sum
             const float x = warp_sum_f32(lane_sum_strided(H_part + (size_t)o * GS, G, lane));
@@ -1019,17 +1021,23 @@ __global__ void __launch_bounds__(STEP_T, 1) k_master_reduce_step(const float* _
 // grid, with one more aperture at intensity 0, is at the point the last one ended
 // on: z, pi, F, g and H of the older apertures stand, and only the new
 // aperture's g and its column of H are formed (MODE_EXT).
-// One plan of 50 apertures, H&N-shaped (304,184 voxels), FP16 storage: 6.71 ms,
+// One plan of 50 apertures, H&N-shaped (304,184 voxels), FP16 storage: 6.64 ms,
 // against 8.70 with blocks of 256 threads on 128-voxel chunks copied by TMA, five
 // block barriers to a chunk, and the step taken by one block between two grid
 // barriers; 8 prostate-shaped plans of 20 apertures at once 8.33 ms (10.96).  An
-// evaluation now takes 22.7 us on average (28 before): tiles 6.4, the update of
-// H 1.6, partials 0.7, waiting for the last block 2.6, reduction and collection
-// 5.2, step 5.0.  The pass is bound by instruction issue, the rest by latency.
-// Every wait is bounded: after GRID_WAIT_LIMIT polls the block reports st->err = 2, marks the barrier broken (later launches of the solve return at
-// entry) and every block leaves at its next wait.
+// evaluation now takes 20.6 us on average (28 before): tiles 6.3, the update of
+// H 1.6, partials 0.7, waiting for the last block 2.5, reduction and collection
+// 4.0, step 5.0.  The pass is bound by instruction issue, the rest by latency.
+// Every wait is bounded: after GRID_WAIT_LIMIT polls the block reports st->err = 2,
+// marks the barrier broken (later launches of the solve return at entry) and every
+// block leaves at its next wait.
 constexpr int PT = 512;            // threads per block (the step takes the first STEP_T)
 constexpr int PW = PT / 32;
+// Up to this many blocks each thread of the step polls its own words at once (20
+// apertures on 19,200 voxels, 38 blocks: 1.93 ms, 1.97 if a warp polls one word
+// first, which is a second trip to L2); on more, their polls keep the L2 from the
+// reducing warps (152 blocks, 50 apertures: 6.70 ms, 6.64 after one word).
+constexpr int DIRECT_BLOCKS = 64;
 constexpr int RING = 21;           // groups of four columns of a tile in a warp's ring
 constexpr int RING_LD = 132;       // floats of a group in the ring: 32 voxels x 4, and 4 against bank conflicts
 constexpr size_t RING_BYTES = (size_t)PW * RING * RING_LD * sizeof(float);
@@ -1610,16 +1618,21 @@ __device__ __forceinline__ void master_solve_group(
             const int v = tid & (KMAX - 1);
             unsigned long long w[KMAX * KMAX / STEP_T], x[5];
             auto waits = [&](int r) { return r < K && v <= r && (mode != MODE_EXT || r == K - 1); };
-            // first one word that the last reducing warps write, until it is there
-            // (every thread polling all its words would keep the L2 from the reducers)
+            // on many blocks first one of the words that take longest, polled by one warp
             int tries = 0;
             auto again = [&]() {
                 if (++tries < GRID_WAIT_LIMIT && ((tries & 4095) || !ld_acquire_gpu(&gb->broken))) return true;
                 s_lost = 1;
                 return false;
             };
-            const unsigned long long* probe = &st->wgn[K - 1];
-            while ((unsigned)(word_get(probe) >> 32) != tag && again()) __nanosleep(40);
+            if (G > DIRECT_BLOCKS) {
+                if (warp == 0) {
+                    const unsigned long long* probe = mode == MODE_EXT ? &st->wg[2 * K - 1] : &st->wF[1];
+                    while ((unsigned)(word_get(probe) >> 32) != tag && again()) {
+                    }
+                }
+                step_sync();
+            }
             for (bool ok = false; !ok;) {
                 ok = true;
 #pragma unroll

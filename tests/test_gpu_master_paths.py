@@ -45,6 +45,8 @@ def _pool(case, n, seed):
     (5000, 1, (3, 4, 9, 10, 14, 20, 21, 28, 40, 41, 44, 45, 64), False, "fp32"),
     (5000, 3, (5, 6, 40, 41), True, "fp16"),
     (9000, 1, (12, 13, 30, 31), False, "fp16"), (9000, 0, (2, 17, 18, 48), True, "fp32"),
+    # polls of a word each or of one word first (from 65 blocks), and blocks without a tile
+    (34000, 64, (3, 4, 40), False, "fp32"), (34000, 65, (3, 4, 40), False, "fp32"), (700, 152, (2, 3, 9), True, "fp32"),
 ])
 def test_master_forms_match_the_oracle(torch, V, blocks, sizes, negative, prec):
     from paper_1003_5402_gb300 import Plan, binding
