@@ -720,7 +720,7 @@ cudaError_t price_any(dao_ctx* c, const float* w, const int* skip, cudaStream_t 
                             n);
     cudaError_t e = price_rows_any(c, w, skip, s, n);
     if (e != cudaSuccess) return e;
-    return launch_price_beams(c->row_v, c->beam_row0_d, c->B, c->price, skip, s, n);
+    return launch_price_beams(c->row_v, c->beam_row0_d, c->B, c->price, skip, s, n, c->R_tot);
 }
 
 // pi = grad F(z) and z at the current pool's accepted intensities (final pass).
@@ -1018,6 +1018,7 @@ bool build_solve_graph_persist(dao_ctx* c) {
             ca.beam_off = c->beam_off_d;
             ca.seg = c->seg;
             ca.n_beams = c->B;
+            ca.n_rows = c->R_tot;
             ca.lr_stride = 2 * c->max_rows;
             ca.tau = c->tau;
             ca.ap_beam = c->ap_beam;
@@ -1583,8 +1584,8 @@ dao_status dao_price(dao_ctx* c, int32_t* beam, int32_t* leaf_lr, double* rc) {
     c->prof_end();
     c->prof_begin(DAO_KC_PRICE);
     if (mlc) DAO_CU(price_rows_any(c, c->w, nullptr, c->stream, &c->launches_i));
-    DAO_CU(launch_price_beams(c->row_v, c->beam_row0_d, c->B, pd, nullptr, c->stream, &c->launches_i, c->row_lr,
-                              reinterpret_cast<int2*>(lr)));
+    DAO_CU(launch_price_beams(c->row_v, c->beam_row0_d, c->B, pd, nullptr, c->stream, &c->launches_i, c->R_tot,
+                              c->row_lr, reinterpret_cast<int2*>(lr)));
     c->prof_end();
     DAO_TRY(sync(c));
     c->count_launches();
@@ -2302,6 +2303,7 @@ dao_status build_batch_graph(dao_ctx* const* ctxs, int n, int R, BatchGraph* bg)
             ca.beam_off = c->beam_off_d;
             ca.seg = c->seg;
             ca.n_beams = c->B;
+            ca.n_rows = c->R_tot;
             ca.lr_stride = 2 * c->max_rows;
             ca.tau = c->tau;
             ca.ap_beam = c->ap_beam;

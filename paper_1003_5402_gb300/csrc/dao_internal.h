@@ -264,11 +264,11 @@ cudaError_t launch_price_commit(const double* row_v, const int* beam_row0, int n
                                 const int2* row_lr, const int* rows, const int* cols, double tau, int K, int lr_stride,
                                 int* ap_beam, int* ap_lr, float* mask, CGDev* cg, cudaStream_t stream, int* launches);
 
-// Only the per-beam sums of row_v and their argmin (k_price_beams), with the best
-// beam's rows of row_lr into leaves when that is given.
+// Only the per-beam sums of row_v (n_rows values) and their argmin (k_price_beams),
+// with the best beam's rows of row_lr into leaves when that is given.
 cudaError_t launch_price_beams(const double* row_v, const int* beam_row0, int n_beams, PriceDev* out,
-                               const int* skip, cudaStream_t stream, int* launches, const int2* row_lr = nullptr,
-                               int2* leaves = nullptr);
+                               const int* skip, cudaStream_t stream, int* launches, int n_rows,
+                               const int2* row_lr = nullptr, int2* leaves = nullptr);
 // a3 under an MLC constraint (mlc.cu): one block per beam writes row_v (the
 // beam's value at its first row, 0 at the others) and row_lr; smem bytes from
 // mlc_smem_bytes for the largest beam, after mlc_configure with that size.
@@ -339,6 +339,8 @@ struct CommitArgs {
     const int* beam_off;
     const int* seg;         // (B + 1) x V beam segments of D's rows
     int n_beams;
+    int n_rows;             // MLC rows of all beams
+    int stage_rows;         // n_rows: the kernel stages their values in shared memory; 0: not (set by the launch)
     int lr_stride;
     double tau;
     int* ap_beam;

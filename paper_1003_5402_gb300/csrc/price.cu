@@ -18,18 +18,28 @@ __global__ void __launch_bounds__(256) k_price_rows(const float* __restrict__ w,
     pricing::row_best(w, row_info[g], g, row_v, row_lr);
 }
 
-// One block: thread b sums beam b's rows in row order; thread 0 takes the argmin.
-// leaves (nullable): the best beam's leaf positions.  out and leaves may be
-// page-locked host memory, which saves the copies after the kernel.
+// One block: the rows' values fetched together into shared memory (stage_rows of
+// them; 0, beyond 40 KB: read where they are, a chain of loads; pricing call of 5
+// beams of 30 x 30: 45.5 us with 16 rows requested ahead, 44.8 staged), thread b sums beam b's rows in row order, thread 0
+// takes the argmin.  leaves (nullable): the best beam's leaf positions.  out and
+// leaves may be page-locked host memory, which saves the copies after the kernel.
 __global__ void __launch_bounds__(256) k_price_beams(const double* __restrict__ row_v,
                                                      const int* __restrict__ beam_row0, int n_beams,
                                                      PriceDev* __restrict__ out, const int2* __restrict__ row_lr,
-                                                     int2* __restrict__ leaves, const int* __restrict__ skip) {
+                                                     int2* __restrict__ leaves, int stage_rows,
+                                                     const int* __restrict__ skip) {
     extern __shared__ double s_sum[];
     __shared__ int s_best;
     if (skip != nullptr && *skip) return;
-    for (int b = threadIdx.x; b < n_beams; b += blockDim.x)
-        s_sum[b] = pricing::beam_sum(row_v, beam_row0[b], beam_row0[b + 1]);
+    double* s_rows = s_sum + n_beams;
+    for (int r = threadIdx.x; r < stage_rows; r += blockDim.x) s_rows[r] = row_v[r];
+    __syncthreads();
+    const double* rv = stage_rows ? s_rows : row_v;
+    for (int b = threadIdx.x; b < n_beams; b += blockDim.x) {
+        double t = 0.0;
+        for (int r = beam_row0[b]; r < beam_row0[b + 1]; ++r) t = t + rv[r];
+        s_sum[b] = t;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         int best = 0;
@@ -117,9 +127,11 @@ cudaError_t launch_price_commit(const double* row_v, const int* beam_row0, int n
 }
 
 cudaError_t launch_price_beams(const double* row_v, const int* beam_row0, int n_beams, PriceDev* out,
-                               const int* skip, cudaStream_t stream, int* launches, const int2* row_lr, int2* leaves) {
-    k_price_beams<<<1, 256, (size_t)(n_beams > 0 ? n_beams : 1) * sizeof(double), stream>>>(
-        row_v, beam_row0, n_beams, out, row_lr, leaves, skip);
+                               const int* skip, cudaStream_t stream, int* launches, int n_rows, const int2* row_lr,
+                               int2* leaves) {
+    const int stage = ((size_t)n_rows + n_beams) * sizeof(double) <= 40 * 1024 ? n_rows : 0;
+    k_price_beams<<<1, 256, (size_t)(n_beams + stage + 1) * sizeof(double), stream>>>(
+        row_v, beam_row0, n_beams, out, row_lr, leaves, stage, skip);
     ++*launches;
     return cudaGetLastError();
 }
@@ -137,7 +149,7 @@ cudaError_t launch_price(const float* w, const int4* row_info, int n_rows, const
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    return launch_price_beams(row_v, beam_row0, n_beams, out, skip, stream, launches);
+    return launch_price_beams(row_v, beam_row0, n_beams, out, skip, stream, launches, n_rows);
 }
 
 }  // namespace dao

@@ -89,40 +89,32 @@ __device__ __forceinline__ void row_best(const float* __restrict__ w, int4 ri, i
     }
 }
 
-// Sum of rows [r0, r1) of row_v in row order, 16 rows requested before the first
-// add (a plain loop waits for L2 at every add).  Not for decide below: there the
-// registers would cost the fused column kernel's occupancy (a plan of 50
-// apertures, H&N-shaped: 7.31 against 6.71 ms).
-__device__ __forceinline__ double beam_sum(const double* __restrict__ row_v, int r0, int r1) {
-    double t = 0.0;
-    for (int r = r0; r < r1; r += 16) {
-        double v[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) v[q] = r + q < r1 ? __ldcg(row_v + r + q) : 0.0;
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-            if (r + q < r1) t = t + v[q];
-    }
-    return t;
-}
-
 enum { OUTCOME_NEW = 0, OUTCOME_OPTIMAL = 1, OUTCOME_DUPLICATE = 2 };
 
 // Whole block (every thread calls it): beam sums into s_sum (n_beams doubles
 // of shared memory), argmin, stop test, then the duplicate test against the
 // K - 1 apertures of the pool.  Every thread returns the same outcome, beam
-// and reduced cost.
+// and reduced cost.  s_rows (nullable): room for the rows' values, which the
+// block then fetches together instead of every beam's thread in a chain of
+// round trips to L2 (a plan of 50 apertures, H&N-shaped: 6.57 against 6.53 ms; rows
+// requested ahead into registers instead cost the fused column kernel its
+// occupancy, 7.31).
 __device__ __forceinline__ int decide(const double* __restrict__ row_v, const int* __restrict__ beam_row0,
                                       int n_beams, const int2* __restrict__ row_lr, const int* __restrict__ rows,
                                       double tau, int K, int lr_stride, const int* __restrict__ ap_beam,
                                       const int* __restrict__ ap_lr, double* s_sum, int* beam_out,
-                                      double* rc_out) {
+                                      double* rc_out, double* s_rows = nullptr) {
     __shared__ int s_best, s_dup;
     __shared__ double s_rc;
     const int tid = threadIdx.x;
+    if (s_rows != nullptr) {
+        for (int r = tid; r < beam_row0[n_beams]; r += blockDim.x) s_rows[r] = row_v[r];
+        __syncthreads();
+    }
+    const double* rv = s_rows != nullptr ? s_rows : row_v;
     for (int b = tid; b < n_beams; b += blockDim.x) {
         double t = 0.0;
-        for (int r = beam_row0[b]; r < beam_row0[b + 1]; ++r) t = t + row_v[r];
+        for (int r = beam_row0[b]; r < beam_row0[b + 1]; ++r) t = t + rv[r];
         s_sum[b] = t;
     }
     __syncthreads();

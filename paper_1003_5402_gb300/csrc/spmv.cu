@@ -919,8 +919,9 @@ __global__ void __launch_bounds__(256) k_commit_column(const int* __restrict__ c
                                                        const float* __restrict__ bval32,
                                                        const unsigned short* __restrict__ bval16) {
     extern __shared__ double s_dyn[];
-    double* s_sum = s_dyn;                                        // n_beams
-    float* smask = reinterpret_cast<float*>(s_dyn + ca.n_beams);  // max_nb
+    double* s_sum = s_dyn;                                                        // n_beams
+    double* s_rows = ca.stage_rows ? s_dyn + ca.n_beams : nullptr;                // MLC rows
+    float* smask = reinterpret_cast<float*>(s_dyn + ca.n_beams + ca.stage_rows);  // max_nb
     CGDev* cg = ca.cg;
     const int tid = threadIdx.x;
     const bool lead = blockIdx.x == 0 && tid == 0;
@@ -939,7 +940,7 @@ __global__ void __launch_bounds__(256) k_commit_column(const int* __restrict__ c
     int b = 0;
     double rc = 0.0;
     const int outcome = pricing::decide(ca.row_v, ca.beam_row0, ca.n_beams, ca.row_lr, ca.rows, ca.tau, K,
-                                        ca.lr_stride, ca.ap_beam, ca.ap_lr, s_sum, &b, &rc);
+                                        ca.lr_stride, ca.ap_beam, ca.ap_lr, s_sum, &b, &rc, s_rows);
     if (outcome != pricing::OUTCOME_NEW) {
         if (lead) cg->done = outcome;
         finish(1, 1);
@@ -1418,11 +1419,16 @@ static void commit_column_launch(const DevCSR& D, const CommitArgs& ca, size_t s
                                                                       D.beam_val32, nullptr);
 }
 
-cudaError_t launch_commit_column(const DevCSR& D, const CommitArgs& ca, int max_nb, int num_sms, cudaStream_t stream,
-                                 int* launches) {
-    if (D.n_rows == 0 || ca.cg == nullptr) return cudaErrorInvalidValue;
+cudaError_t launch_commit_column(const DevCSR& D, const CommitArgs& args, int max_nb, int num_sms,
+                                 cudaStream_t stream, int* launches) {
+    if (D.n_rows == 0 || args.cg == nullptr) return cudaErrorInvalidValue;
     const int grid = num_sms * 8;
-    const size_t sm = (size_t)std::max(ca.n_beams, 1) * sizeof(double) + (size_t)std::max(max_nb, 1) * sizeof(float);
+    CommitArgs ca = args;
+    size_t sm = (size_t)std::max(ca.n_beams, 1) * sizeof(double) + (size_t)std::max(max_nb, 1) * sizeof(float);
+    // the rows' values in shared memory too, while eight blocks per SM still fit
+    ca.stage_rows = ca.n_rows;
+    if (sm + (size_t)ca.n_rows * sizeof(double) > 24 * 1024) ca.stage_rows = 0;
+    sm += (size_t)ca.stage_rows * sizeof(double);
     if (column_by_beams(D)) {
         commit_column_launch<0>(D, ca, sm, grid, stream);
         ++*launches;
