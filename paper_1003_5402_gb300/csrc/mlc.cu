@@ -34,6 +34,12 @@ namespace dao {
 namespace {
 
 constexpr int MLC_THREADS = 256;
+// Interdigitation: each MLC row's step takes two tables of prefix minima (at most 33
+// lines of 33), a warp to a line.  A thread to a line walks 33 dependent
+// comparisons: the pricing call of 9 beams of 20 x 20 took 98 us so, 79 with a warp
+// scanning each line.
+constexpr int MLC_THREADS_IL = 1024;
+constexpr int mlc_threads(int mode) { return mode == DAO_MLC_INTERDIGITATION ? MLC_THREADS_IL : MLC_THREADS; }
 
 // A double as an integer that orders like it (a NaN above infinity, so that it is
 // never the smaller; -0 as 0): the dynamic programme's minima are chains of
@@ -60,6 +66,21 @@ __device__ __forceinline__ bool mlc_better(mlc_key v, int i, mlc_key bv, int bi)
 // index of the leaf state (L, R), 0 <= L <= R <= C (C1 = C + 1), L-major
 __device__ __forceinline__ int mlc_state(int L, int R, int C1) { return L * C1 - L * (L - 1) / 2 + (R - L); }
 
+// Inclusive running minimum over the warp's lanes of (value, index): by value, the
+// smaller index on equal ones, so the same in whatever order the scan combines.
+__device__ __forceinline__ void mlc_scan(mlc_key& m, int& mi) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const mlc_key om = __shfl_up_sync(0xffffffffu, m, o);
+        const int oi = __shfl_up_sync(0xffffffffu, mi, o);
+        if (lane >= o && mlc_better(om, oi, m, mi)) {
+            m = om;
+            mi = oi;
+        }
+    }
+}
+
 // The paper's one-pass search (Sec. 2.3) over n values v(1..n): running sum,
 // largest running sum with its earliest position, best difference with the
 // earliest end; returns v* and the block [a, b) (v* = 0: none).
@@ -85,7 +106,7 @@ __device__ __forceinline__ double mlc_row_search(int n, Get get, int* a, int* b)
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(MLC_THREADS) k_price_mlc(const float* __restrict__ w,
+__global__ void __launch_bounds__(mlc_threads(MODE)) k_price_mlc(const float* __restrict__ w,
                                                            const int* __restrict__ beam_off,
                                                            const int* __restrict__ rows,
                                                            const int* __restrict__ cols,
@@ -94,7 +115,9 @@ __global__ void __launch_bounds__(MLC_THREADS) k_price_mlc(const float* __restri
                                                            const int* __restrict__ skip) {
     extern __shared__ __align__(16) double sm[];
     if (skip != nullptr && *skip) return;
-    const int b = blockIdx.x, tid = threadIdx.x;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    (void)lane;
+    (void)warp;
     const int R = rows[b], C = cols[b], C1 = C + 1, off = beam_off[b], r0 = beam_row0[b];
     double* P = sm;  // [R][C1]
     // the rows' prices, converted by all threads; then their sums in column order
@@ -120,8 +143,8 @@ __global__ void __launch_bounds__(MLC_THREADS) k_price_mlc(const float* __restri
         unsigned short* back = reinterpret_cast<unsigned short*>(Gi + C1 * C1);  // [R][NS]
         unsigned char* sL = reinterpret_cast<unsigned char*>(back + R * NS);     // [NS]
         unsigned char* sR = sL + NS;                                            // [NS]
-        __shared__ mlc_key s_key[MLC_THREADS / 32];
-        __shared__ int s_idx[MLC_THREADS / 32];
+        __shared__ mlc_key s_key[MLC_THREADS_IL / 32];
+        __shared__ int s_idx[MLC_THREADS_IL / 32];
         __shared__ unsigned short s_path[64];  // the rows' states (at most 64 rows)
         for (int L = tid; L <= C; L += blockDim.x)
             for (int Rr = L; Rr <= C; ++Rr) {
@@ -133,41 +156,59 @@ __global__ void __launch_bounds__(MLC_THREADS) k_price_mlc(const float* __restri
         for (int s = tid; s < NS; s += blockDim.x) f[s] = mlc_to_key(P[sR[s]] - P[sL[s]]);
         __syncthreads();
         for (int r = 1; r < R; ++r) {
-            // H[a][x] = min over R >= max(a, x) of f(a, R)
-            for (int a = tid; a <= C; a += blockDim.x) {
+            // H[a][x] = min over R >= max(a, x) of f(a, R): a warp per a, lane l
+            // the entry R = C - l (and, of 33 entries, lane 31 also R = 0)
+            for (int a = warp; a <= C; a += MLC_THREADS_IL / 32) {
+                const int s0 = mlc_state(a, a, C1) - a, Rr = C - lane;
                 mlc_key m = MLC_KEY_INF;
                 int mi = INT_MAX;
-                const int s0 = mlc_state(a, a, C1) - a;
-#pragma unroll 4
-                for (int Rr = C; Rr >= a; --Rr) {
-                    const mlc_key v = f[s0 + Rr];
-                    if (mlc_better(v, s0 + Rr, m, mi)) {
-                        m = v;
-                        mi = s0 + Rr;
-                    }
+                if (Rr >= a && mlc_better(f[s0 + Rr], s0 + Rr, m, mi)) {
+                    m = f[s0 + Rr];
+                    mi = s0 + Rr;
+                }
+                mlc_scan(m, mi);
+                if (Rr >= a) {
                     Gv[a * C1 + Rr] = m;
                     Gi[a * C1 + Rr] = mi;
                 }
-                for (int x = a - 1; x >= 0; --x) {
-                    Gv[a * C1 + x] = m;
-                    Gi[a * C1 + x] = mi;
+                // below a the value at R = a stands
+                const mlc_key ma = __shfl_sync(0xffffffffu, m, min(C - a, 31));
+                const int ia = __shfl_sync(0xffffffffu, mi, min(C - a, 31));
+                if (lane < a) {
+                    Gv[a * C1 + lane] = ma;
+                    Gi[a * C1 + lane] = ia;
+                }
+                if (C == 32 && a == 0 && lane == 31) {  // R = 0 after R = 1
+                    const bool b0 = mlc_better(f[s0], s0, m, mi);
+                    Gv[0] = b0 ? f[s0] : m;
+                    Gi[0] = b0 ? s0 : mi;
                 }
             }
             __syncthreads();
-            // G[a][x] = min over a' <= a of H[a'][x]: min over L <= a, R >= x
-            for (int x = tid; x <= C; x += blockDim.x) {
+            // G[a][x] = min over a' <= a of H[a'][x]: min over L <= a, R >= x; a warp
+            // per x, lane l the entry a = l (and, of 33 entries, lane 31 also a = 32)
+            for (int x = warp; x <= C; x += MLC_THREADS_IL / 32) {
                 mlc_key m = MLC_KEY_INF;
                 int mi = INT_MAX;
-#pragma unroll 4
-                for (int a = 0; a <= C; ++a) {
-                    const mlc_key v = Gv[a * C1 + x];
-                    const int i = Gi[a * C1 + x];
+                if (lane <= C) {
+                    const mlc_key v = Gv[lane * C1 + x];
+                    const int i = Gi[lane * C1 + x];
                     if (mlc_better(v, i, m, mi)) {
                         m = v;
                         mi = i;
                     }
-                    Gv[a * C1 + x] = m;
-                    Gi[a * C1 + x] = mi;
+                }
+                mlc_scan(m, mi);
+                if (lane <= C) {
+                    Gv[lane * C1 + x] = m;
+                    Gi[lane * C1 + x] = mi;
+                }
+                if (C == 32 && lane == 31) {
+                    const mlc_key v = Gv[32 * C1 + x];
+                    const int i = Gi[32 * C1 + x];
+                    const bool b0 = mlc_better(v, i, m, mi);
+                    Gv[32 * C1 + x] = b0 ? v : m;
+                    Gi[32 * C1 + x] = b0 ? i : mi;
                 }
             }
             __syncthreads();
@@ -208,7 +249,7 @@ __global__ void __launch_bounds__(MLC_THREADS) k_price_mlc(const float* __restri
         if (tid == 0) {
             mlc_key m = s_key[0];
             int best = s_idx[0];
-            for (int q = 1; q < MLC_THREADS / 32; ++q)
+            for (int q = 1; q < MLC_THREADS_IL / 32; ++q)
                 if (mlc_better(s_key[q], s_idx[q], m, best)) {
                     m = s_key[q];
                     best = s_idx[q];
@@ -307,7 +348,7 @@ __global__ void __launch_bounds__(MLC_THREADS) k_price_mlc(const float* __restri
 template <int MODE>
 cudaError_t mlc_launch(const float* w, const int* beam_off, const int* rows, const int* cols, const int* beam_row0,
                        int n_beams, size_t smem, double* row_v, int2* row_lr, const int* skip, cudaStream_t stream) {
-    k_price_mlc<MODE><<<n_beams, MLC_THREADS, smem, stream>>>(w, beam_off, rows, cols, beam_row0, row_v, row_lr,
+    k_price_mlc<MODE><<<n_beams, mlc_threads(MODE), smem, stream>>>(w, beam_off, rows, cols, beam_row0, row_v, row_lr,
                                                               skip);
     return cudaGetLastError();
 }
