@@ -23,7 +23,7 @@ constexpr int NA_MAX_BLOCKS = 1024;      // size of the scratch array
 constexpr int NA_THREADS = 512;
 constexpr int NA_WARPS = NA_THREADS / 32;
 constexpr int NA_CHUNK = 1024;           // products a warp holds at a time
-constexpr int NA_AHEAD = 8;              // entries per lane requested together
+constexpr int NA_AHEAD = 6;              // entries per lane requested together
 constexpr int NA_MAX_DEVICES = 64;
 constexpr int SMAX_TERMS = dao::SMAX;
 
@@ -58,7 +58,8 @@ __device__ __forceinline__ double na_block_sum(double v, double* s_red) {
 
 // A warp takes units of 32 consecutive rows (grid-stride): their entries are one
 // contiguous range, read with consecutive entries on consecutive lanes, NA_AHEAD
-// per lane in flight; the products go to the warp's chunk of shared memory, and
+// per lane in flight, the next ones (and the next unit's row offsets) requested
+// before these are used; the products go to the warp's chunk of shared memory, and
 // lane r sums row r's from there (four interleaved partial sums), so that every
 // lane then has a row of its own for the FP64 epilogue.  The caller's rows have
 // no padding, so wider loads would start off their alignment.  X: x in shared
@@ -69,7 +70,8 @@ __device__ __forceinline__ double na_block_sum(double v, double* s_red) {
 // (304,184 voxels, 9.55 M entries).  With 8 lanes to a row the epilogue's FP64
 // instructions (1/64 of the FP32 rate) ran with four lanes of 32 in use and each
 // lane waited for its gather before its next entry: 104 us; the call took 158 us
-// and takes 85 now, of which the kernel is the smaller part.
+// and takes 84 now (85.8 without the requests ahead), of which the kernel is the
+// smaller part.
 template <bool X>
 __global__ void __launch_bounds__(NA_THREADS, 2) k_dose_noalloc(int V, int N, const int* __restrict__ rowptr,
                                                                const int* __restrict__ col,
@@ -83,6 +85,7 @@ __global__ void __launch_bounds__(NA_THREADS, 2) k_dose_noalloc(int V, int N, co
     extern __shared__ float s_na[];
     __shared__ double s_red[NA_WARPS];
     __shared__ double s_t[SMAX_TERMS][4];
+    __shared__ float2 s_f[SMAX_TERMS];  // T^- rounded up, T^+ rounded down: an FP32 z compares with these as with the FP64
     __shared__ int s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* buf = s_na + warp * NA_CHUNK;
@@ -93,29 +96,51 @@ __global__ void __launch_bounds__(NA_THREADS, 2) k_dose_noalloc(int V, int N, co
     for (int i = threadIdx.x; i < 4 * S && busy; i += NA_THREADS) {
         const double t = (&terms.t[0][0])[i];
         (&s_t[0][0])[i] = t;
+        if ((i & 3) == 1) s_f[i >> 2].x = __double2float_ru(t);
+        if ((i & 3) == 3) s_f[i >> 2].y = __double2float_rd(t);
         fin = fin && isfinite(t);
     }
     if (X && busy)
         for (int i = threadIdx.x; i < N; i += NA_THREADS) sx[i] = __ldg(x + i);
     const bool finite = __syncthreads_and(fin) != 0;
     double facc = 0.0;
-    for (int u = blockIdx.x * NA_WARPS + warp; u < units; u += gridDim.x * NA_WARPS) {
+    int rs_n = 0, re_n = 0, lab_n = 0;  // the next unit's row offsets and labels, requested ahead
+    auto unit_in = [&](int u) {
+        const int row = min(u, units) * 32 + lane;
+        rs_n = __ldg(rowptr + min(row, V));
+        re_n = __ldg(rowptr + min(row + 1, V));
+        lab_n = row < V ? __ldg(vstruct + row) : 0;
+    };
+    const int u0 = blockIdx.x * NA_WARPS + warp;
+    if (u0 < units) unit_in(u0);
+    for (int u = u0; u < units; u += gridDim.x * NA_WARPS) {
         const int row = u * 32 + lane;
-        const int rs = __ldg(rowptr + min(row, V)), re = __ldg(rowptr + min(row + 1, V));
-        const int lab = row < V ? __ldg(vstruct + row) : 0;
+        const int rs = rs_n, re = re_n, lab = lab_n;
+        unit_in(u + gridDim.x * NA_WARPS);
         const int e0 = __shfl_sync(0xffffffffu, rs, 0), e1 = __shfl_sync(0xffffffffu, re, 31);
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
         for (int c0 = e0; c0 < e1; c0 += NA_CHUNK) {
             const int c1 = min(e1, c0 + NA_CHUNK);
+            int cn[NA_AHEAD];
+            float vn[NA_AHEAD];
+            auto batch_in = [&](int p0) {
+#pragma unroll
+                for (int q = 0; q < NA_AHEAD; ++q) {
+                    const int p = p0 + 32 * q + lane;
+                    cn[q] = p < c1 ? __ldg(col + p) : 0;
+                    vn[q] = p < c1 ? __ldg(val + p) : 0.f;
+                }
+            };
+            batch_in(c0);
             for (int p0 = c0; p0 < c1; p0 += 32 * NA_AHEAD) {
                 int c[NA_AHEAD];
                 float v[NA_AHEAD];
 #pragma unroll
                 for (int q = 0; q < NA_AHEAD; ++q) {
-                    const int p = p0 + 32 * q + lane;
-                    c[q] = p < c1 ? __ldg(col + p) : 0;
-                    v[q] = p < c1 ? __ldg(val + p) : 0.f;
+                    c[q] = cn[q];
+                    v[q] = vn[q];
                 }
+                batch_in(p0 + 32 * NA_AHEAD);
 #pragma unroll
                 for (int q = 0; q < NA_AHEAD; ++q) {
                     const int p = p0 + 32 * q + lane;
@@ -141,12 +166,11 @@ __global__ void __launch_bounds__(NA_THREADS, 2) k_dose_noalloc(int V, int N, co
                 if (grad != nullptr) grad[row] = __int_as_float(0x7fc00000);
                 facc += __longlong_as_double(0x7ff8000000000000ll);  // the objective becomes NaN
             } else {
-                const double* tt = s_t[lab];
-                const double zd = zr;
-                const double du = tt[1] - zd, dv = zd - tt[3];
                 float g = 0.f;
-                if (du > 0.0 || dv > 0.0 || !finite) {  // else both penalties are 0 (so most voxels)
-                    const double uu = fmax(0.0, du), o = fmax(0.0, dv);
+                if (zr < s_f[lab].x || zr > s_f[lab].y || !finite) {  // else both penalties are 0 (so most voxels)
+                    const double* tt = s_t[lab];
+                    const double zd = zr;
+                    const double uu = fmax(0.0, tt[1] - zd), o = fmax(0.0, zd - tt[3]);
                     g = (float)(2.0 * (tt[2] * o - tt[0] * uu));
                     facc += tt[0] * uu * uu + tt[2] * o * o;
                 }
