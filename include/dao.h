@@ -130,8 +130,8 @@ typedef struct dao_options {
     int32_t master_blocks;     /* blocks of the persistent master solve; 0 (default): one per SM, or fewer
                                 * where they give every warp its voxels; n > 0: n blocks (at most one per SM),
                                 * which leaves room for other plans' solves to run side by side */
-    int32_t dt_threads;        /* threads per beamlet row of the transposed SpMV: 0 (default: 64, or the
-                                * autotuner's choice), 64, 128 or 256 */
+    int32_t dt_threads;        /* threads per beamlet row of the transposed SpMV: 0 (default: 128 in the
+                                * consecutive form of FP32 storage, else 64, or the autotuner's choice), 64, 128 or 256 */
     int32_t dt_map;            /* form of the transposed SpMV: 0 (default: DAO_DT_CONSECUTIVE, or the
                                 * autotuner's choice); DAO_DT_GROUPED (a block per beamlet row, a thread per
                                 * 4 or 8 consecutive entries, 16-byte loads), DAO_DT_CONSECUTIVE (a block per

@@ -2428,7 +2428,7 @@ dao_status dao_kernel_forms(const dao_ctx* c, dao_tuning* out) {
     out->dose_lanes = D.tune_dose_g;
     out->column_lanes = D.tune_col_g;  // 0: the beam layout
     out->dt_map = split ? DT_MAP_SPLIT : Dt.tune_dt_map == DT_MAP_GROUPED ? DT_MAP_GROUPED : DT_MAP_CONSECUTIVE;
-    out->dt_threads = split ? 0 : (Dt.tune_dt_threads ? Dt.tune_dt_threads : 64);
+    out->dt_threads = split ? 0 : (Dt.tune_dt_threads ? Dt.tune_dt_threads : dt_threads_default(Dt));
     out->from_cache = 0;
     return DAO_OK;
 }

@@ -127,6 +127,18 @@ constexpr int MERGE_CHUNK_MAX = 1024;
 // Lane mappings of the transposed SpMV (a2): a thread per group of 4 or 8
 // consecutive entries, or consecutive entries on consecutive threads (default).
 enum { DT_MAP_GROUPED = DAO_DT_GROUPED, DT_MAP_CONSECUTIVE = DAO_DT_CONSECUTIVE, DT_MAP_SPLIT = DAO_DT_SPLIT };
+
+// Threads of the block-per-row transposed SpMV when none are asked for.  64 keep
+// every row of a few thousand resident in one wave; 128 halve the longest row's
+// chain of batches, which pays with FP32 values: k_beamlet_prices on an H&N-shaped
+// matrix 31.2 -> 29.8 us, pricing call of a prostate-shaped one 78.1 -> 76.3, plan
+// on 500 rows 1.928 -> 1.911 ms.  With 16-bit values it does not (8 prostate-shaped
+// plans at once 8.28 -> 8.65 ms, H&N-shaped pricing call 44.9 -> 45.6 us, prices of
+// 2380 rows 17.8 -> 19.1).
+inline int dt_threads_default(const DevCSR& Dt) {
+    if (Dt.tune_dt_map == DT_MAP_GROUPED) return 64;
+    return Dt.prec == DAO_PREC_FP32 ? 128 : 64;
+}
 // Warps of the split form of a2 per SM (blocks of 8 warps).
 constexpr int SPLIT_WARPS_PER_SM = 32;
 

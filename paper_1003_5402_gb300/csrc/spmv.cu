@@ -1273,12 +1273,11 @@ static cudaError_t dt_dispatch(const DevCSR& Dt, const float* pi, float* w, cons
         ++*launches;
         return cudaGetLastError();
     }
-    // one block per beamlet row; 64 threads by default, so that up to 32 blocks
-    // per SM keep every row resident in one wave
-    switch (Dt.tune_dt_threads) {
-        case 128: dt_launch_map<128>(Dt, pi, w, skip, rt, stream); break;
+    // one block per beamlet row
+    switch (Dt.tune_dt_threads ? Dt.tune_dt_threads : dt_threads_default(Dt)) {
+        case 64: dt_launch_map<64>(Dt, pi, w, skip, rt, stream); break;
         case 256: dt_launch_map<256>(Dt, pi, w, skip, rt, stream); break;
-        default: dt_launch_map<64>(Dt, pi, w, skip, rt, stream); break;
+        default: dt_launch_map<128>(Dt, pi, w, skip, rt, stream); break;
     }
     ++*launches;
     return cudaGetLastError();
