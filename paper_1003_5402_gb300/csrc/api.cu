@@ -440,8 +440,8 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
     }
     DAO_TRY(cu(build_stats(t_rp, t_col, t_val, V, CH, N, n_ch, t_C, t_cnt, reinterpret_cast<unsigned*>(scale), t_dmax,
                            c->num_sms, st), "transpose counts and scales"));
-    DAO_TRY(cu(build_fill_d(prec, t_rp, t_col, t_val, c->D.rowptr, V, scale, c->D, st), "padded D"));
-    DAO_TRY(cu(build_seg(t_rp, t_col, c->D.rowptr, V, c->beam_off_d, B, c->seg, st), "beam segments"));
+    DAO_TRY(cu(build_fill_d(prec, t_rp, t_col, t_val, c->D.rowptr, V, scale, c->beam_off_d, B, c->seg, c->D, st),
+               "padded D and beam segments"));
     // D by beams for the aperture column (a4): each beam's part of every row
     // in one contiguous range
     DAO_TRY(c->dalloc(&c->D.beam_rowptr, (size_t)B * (V + 1)));
@@ -548,8 +548,7 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
         DAO_TRY(c->dalloc(&c->Dt.val16, tpadded));
         DAO_TRY(talloc(&t_tval, sizeof(float) * tpadded));
     }
-    DAO_TRY(cu(build_transpose_place(prec, t_rp, t_col, t_val, V, CH, N, n_ch, t_C, t_cnt, scale, c->Dt, t_tval,
-                                     c->num_sms, st),
+    DAO_TRY(cu(build_transpose_place(prec, t_rp, t_col, t_val, V, CH, N, n_ch, t_C, t_cnt, scale, c->Dt, t_tval, st),
                "transpose"));
     free_temps();
     float dmax = 0.f;

@@ -8,9 +8,14 @@
 // sequential counting sort gives, without sorting: the voxel rows are cut into
 // chunks; C[chunk][i] counts chunk's entries of beamlet i (shared-memory
 // integer atomics, so the counts are exact); a scan over chunks turns the
-// counts into each chunk's first slot in every row of D^T; then one warp per
-// chunk walks its entries in CSR order and places each at its beamlet's next
-// slot, lanes that share a beamlet taking consecutive slots in lane order.
+// counts into each chunk's first slot in every row of D^T; then a block per
+// chunk places its entries, each at its beamlet's first slot plus the number of
+// the chunk's earlier rows that hold the beamlet, counted in a bitmap of rows.
+//
+// The passes over the entries are bound by latency, not by bytes, unless each
+// warp keeps many loads in flight.  They therefore give a warp several consecutive
+// rows whose entries it reads as one stretch, several per lane requested
+// together, with each lane keeping track of the row that its entry is in.
 #include <algorithm>
 #include <climits>
 
@@ -52,60 +57,102 @@ __global__ void k_scale_fix(unsigned* __restrict__ smax, int N, unsigned* __rest
     }
 }
 
-// Padded voxel-major D, one warp per voxel row; padding repeats the row's last
-// column with value 0.
+constexpr int RW_T = 256, RW_W = RW_T / 32;  // threads and warps of a block
+constexpr int RW_ROWS = 8;                   // rows per warp: with 32 the warps of the longest rows end last
+constexpr int RW_U = 4;                      // entries per lane requested together
+
+// Padded voxel-major D (padding repeats the row's last column with value 0) and
+// its beam segments: seg[b][j] = first padded position of row j with column >=
+// beam_off[b], seg[B][j] = the end of row j's real entries.  A warp per RW_ROWS
+// rows; the segments by a binary search per (row, beam) over columns that the warp
+// has just read.  Prostate-shaped FP32 matrix (7.4 M entries, 9 beams): a warp per
+// row, and a thread per row that walked it again for the segments, took 38 + 49 us;
+// with a search for every entry's beam 59, bound by issue; now 31.
 template <int PREC>
-__global__ void k_fill_d(const int64_t* __restrict__ rp, const int* __restrict__ col, const float* __restrict__ val,
-                         const int* __restrict__ prow, int V, const float* __restrict__ scale,
-                         int* __restrict__ dcol, float* __restrict__ dval, unsigned short* __restrict__ dcol16,
-                         unsigned short* __restrict__ dval16) {
-    const int lane = threadIdx.x & 31;
-    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (j >= V) return;
-    const int64_t p0 = rp[j];
-    const int len = (int)(rp[j + 1] - p0);
-    const int q0 = prow[j], n = prow[j + 1] - q0;
-    const int last = len > 0 ? col[p0 + len - 1] : 0;
-    for (int t = lane; t < n; t += 32) {
-        const int c = t < len ? col[p0 + t] : last;
-        const float v = t < len ? val[p0 + t] : 0.f;
+__global__ void __launch_bounds__(RW_T) k_fill_d(const int64_t* __restrict__ rp, const int* __restrict__ col,
+                                                 const float* __restrict__ val, const int* __restrict__ prow, int V,
+                                                 const float* __restrict__ scale, const int* __restrict__ beam_off,
+                                                 int B, int* __restrict__ seg, int* __restrict__ dcol,
+                                                 float* __restrict__ dval, unsigned short* __restrict__ dcol16,
+                                                 unsigned short* __restrict__ dval16) {
+    __shared__ int s_start[RW_W][RW_ROWS + 1], s_shift[RW_W][RW_ROWS + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w = (int64_t)blockIdx.x * RW_W + warp;
+    if (w * RW_ROWS >= V) return;
+    const int j0 = (int)(w * RW_ROWS), j = min(j0 + min(lane, RW_ROWS), V);  // lane RW_ROWS: the end
+    const bool own = lane < RW_ROWS && j < V;
+    const int64_t p0 = rp[j], s0 = __shfl_sync(FULL, p0, 0);
+    const int len = own ? (int)(rp[j + 1] - p0) : 0;
+    const int q0 = prow[j], pl = own ? prow[j + 1] - q0 : 0;
+    if (lane <= RW_ROWS) {
+        s_start[warp][lane] = (int)(p0 - s0);
+        s_shift[warp][lane] = q0 - (int)(p0 - s0);
+    }
+    __syncwarp();
+    auto put = [&](int q, int c, float v) {
         if (PREC == DAO_PREC_FP32) {
-            dcol[q0 + t] = c;
-            dval[q0 + t] = v;
+            dcol[q] = c;
+            dval[q] = v;
         } else {
-            dcol16[q0 + t] = (unsigned short)c;
-            dval16[q0 + t] = to16<PREC>(v / scale[c]);
+            dcol16[q] = (unsigned short)c;
+            dval16[q] = to16<PREC>(v / scale[c]);
+        }
+    };
+    const int n = s_start[warp][RW_ROWS];
+    int r = 0;  // the row of the lane's entry
+    for (int t0 = 0; t0 < n; t0 += 32 * RW_U) {
+        int c[RW_U];
+        float v[RW_U];
+#pragma unroll
+        for (int u = 0; u < RW_U; ++u) {
+            const int t = t0 + 32 * u + lane;
+            c[u] = t < n ? col[s0 + t] : 0;
+            v[u] = t < n ? val[s0 + t] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < RW_U; ++u) {
+            const int t = t0 + 32 * u + lane;
+            if (t < n) {
+                while (t >= s_start[warp][r + 1]) ++r;
+                put(s_shift[warp][r] + t, c[u], v[u]);
+            }
         }
     }
-}
-
-// seg[b][j] = first padded position of row j with column >= beam_off[b];
-// seg[B][j] = the end of row j's real entries.
-__global__ void k_seg(const int64_t* __restrict__ rp, const int* __restrict__ col, const int* __restrict__ prow,
-                      int V, const int* __restrict__ beam_off, int B, int* __restrict__ seg) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= V) return;
-    const int64_t p0 = rp[j];
-    const int len = (int)(rp[j + 1] - p0);
-    const int q0 = prow[j];
-    int t = 0;
-    for (int b = 0; b < B; ++b) {
-        const int lo = beam_off[b];
-        while (t < len && col[p0 + t] < lo) ++t;
-        seg[(size_t)b * V + j] = q0 + t;
+    if (own) {
+        const int last = len > 0 ? col[p0 + len - 1] : 0;
+        for (int t = len; t < pl; ++t) put(q0 + t, last, 0.f);
     }
-    seg[(size_t)B * V + j] = q0 + len;
+    for (int i = lane; i < RW_ROWS * (B + 1); i += 32) {
+        const int rr = i % RW_ROWS, b = i / RW_ROWS;
+        if (j0 + rr >= V) continue;
+        const int a = s_start[warp][rr];
+        int lo = a, hi = s_start[warp][rr + 1];
+        if (b == B) {
+            lo = hi;
+        } else {
+            const int first = beam_off[b];
+            while (lo < hi) {
+                const int m = (lo + hi) >> 1;
+                if (col[s0 + m] < first)
+                    lo = m + 1;
+                else
+                    hi = m;
+            }
+        }
+        seg[(size_t)b * V + j0 + rr] = s_shift[warp][rr] + lo;
+    }
 }
 
 // Beamlet counters of one block live in shared memory for a tile of TILE_N
 // beamlets; a matrix with more beamlets runs a grid of (chunk, tile) blocks.
 constexpr int TILE_N = 12288;
-constexpr int STATS_T = 256;
+constexpr int STATS_T = 512, STATS_U = 8;
 
 // Per (chunk, beamlet tile): C[chunk][i] = the chunk's entries of beamlet i,
 // counted in shared memory, and s_i = max |D_ij| over them folded into smax
-// (bits of a non-negative float, ordered like the floats) with one atomicMax
-// per beamlet the chunk touches.
+// (bits of a non-negative float, ordered like the floats).  Both maxima only grow,
+// so a value that is not above the one read needs no atomic.  STATS_U entries per
+// thread in flight: 65 us with one on a prostate-shaped FP32 matrix, now 24.
 __global__ void __launch_bounds__(STATS_T) k_chunk_stats(const int64_t* __restrict__ rp, const int* __restrict__ col,
                                                          const float* __restrict__ val, int V, int CH, int N,
                                                          int* __restrict__ C, unsigned* __restrict__ smax) {
@@ -117,19 +164,29 @@ __global__ void __launch_bounds__(STATS_T) k_chunk_stats(const int64_t* __restri
     for (int t = threadIdx.x; t < 2 * nt; t += STATS_T) s_stats[t] = 0u;
     __syncthreads();
     const int64_t p0 = rp[(int64_t)ch * CH], p1 = rp[min((int64_t)V, (int64_t)(ch + 1) * CH)];
-    for (int64_t p = p0 + threadIdx.x; p < p1; p += STATS_T) {
-        const int c = col[p] - i0;
-        if (c >= 0 && c < nt) {
-            atomicAdd(&s_cnt[c], 1u);
-            atomicMax(&s_mx[c], __float_as_uint(fabsf(val[p])));
+    for (int64_t q = p0; q < p1; q += STATS_T * STATS_U) {
+        int c[STATS_U];
+        float v[STATS_U];
+#pragma unroll
+        for (int u = 0; u < STATS_U; ++u) {
+            const int64_t p = q + u * STATS_T + threadIdx.x;
+            c[u] = p < p1 ? col[p] - i0 : -1;
+            v[u] = p < p1 ? val[p] : 0.f;
         }
+#pragma unroll
+        for (int u = 0; u < STATS_U; ++u)
+            if (c[u] >= 0 && c[u] < nt) {
+                const unsigned m = __float_as_uint(fabsf(v[u]));
+                atomicAdd(&s_cnt[c[u]], 1u);
+                if (m > *(volatile unsigned*)&s_mx[c[u]]) atomicMax(&s_mx[c[u]], m);
+            }
     }
     __syncthreads();
     int* Cc = C + (size_t)ch * N + i0;
     for (int t = threadIdx.x; t < nt; t += STATS_T) {
         const unsigned n = s_cnt[t];
         Cc[t] = (int)n;
-        if (n) atomicMax(&smax[i0 + t], s_mx[t]);
+        if (n && s_mx[t] > __ldcg(&smax[i0 + t])) atomicMax(&smax[i0 + t], s_mx[t]);
     }
 }
 
@@ -160,68 +217,103 @@ __global__ void __launch_bounds__(1024) k_chunk_scan(int* __restrict__ C, int n_
     }
 }
 
-// Placement: one warp per (chunk, beamlet tile of width tw) walks the chunk's
-// voxel rows in order, the lanes over a row's entries (distinct beamlets, so no
-// two lanes share a counter).  The next slot of each beamlet of the tile is a
-// shared-memory counter (row start of D^T + the chunk's offset).  Row starts
-// (PL_ROWS rows at a time) and entries (PL_STG at a time) are staged in shared
-// memory with coalesced loads; a row that straddles two stages is finished in
-// the second.  The walk is a chain of shared-memory round trips per row, so
-// the tiles are made narrow enough for about 24 warps per SM.
-constexpr int PL_ROWS = 256, PL_STG = 512;
+// Placement: a block per (chunk, beamlet tile of width tw) takes PL_ROWS voxel rows
+// at a time: a bitmap of the rows that hold each beamlet (PL_ROWS bits in words of
+// 32 rows, word-major so that consecutive beamlets lie in consecutive banks), then
+// each entry at its beamlet's next slot plus the bits below its row, which is the
+// order of a walk in CSR order without the walk.  Equal stretches of entries per warp,
+// PL_U entries per lane requested together; the second reading of the columns
+// comes from cache.  A warp per (chunk, narrower tile) that walked the rows one
+// after another took 198 us on a prostate-shaped FP32 matrix (7.4 M entries, 3600
+// beamlets); now 128, bound by the scattered 4-byte writes.
+constexpr int PL_T = 1024, PL_ROWS = 256, PL_WORDS = PL_ROWS / 32, PL_U = 8;
+constexpr int PL_TILE = 6000;  // beamlets per tile: 36 bytes of shared memory each
 
-__global__ void __launch_bounds__(32) k_chunk_place(const int64_t* __restrict__ rp, const int* __restrict__ col,
-                                                    const float* __restrict__ val, int V, int CH, int N, int tw,
-                                                    const int* __restrict__ C, const int* __restrict__ trow,
-                                                    int* __restrict__ tcol, float* __restrict__ tval) {
+size_t place_smem(int tw) { return sizeof(int) * (size_t)tw * (PL_WORDS + 1); }
+
+__global__ void __launch_bounds__(PL_T) k_chunk_place(const int64_t* __restrict__ rp, const int* __restrict__ col,
+                                                      const float* __restrict__ val, int V, int CH, int N, int tw,
+                                                      const int* __restrict__ C, const int* __restrict__ trow,
+                                                      int* __restrict__ tcol, float* __restrict__ tval) {
     extern __shared__ int s_pl[];
+    __shared__ int s_row[PL_ROWS + 1];  // row starts, relative to the window's first entry
     const int ch = blockIdx.x, i0 = blockIdx.y * tw;
     const int nt = min(tw, N - i0);
-    int* s_slot = s_pl;                   // nt next slots
-    int* s_row = s_slot + nt;             // PL_ROWS + 1 row starts, relative to the window's first entry
-    int* s_col = s_row + PL_ROWS + 1;     // PL_STG staged entries: beamlet - i0
-    float* s_val = reinterpret_cast<float*>(s_col + PL_STG);
-    const int lane = threadIdx.x;
-    for (int t = lane; t < nt; t += 32) s_slot[t] = trow[i0 + t] + C[(size_t)ch * N + i0 + t];
+    int* s_slot = s_pl;                                          // next slots
+    unsigned* s_bits = reinterpret_cast<unsigned*>(s_pl) + tw;   // PL_WORDS x tw
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int t = tid; t < nt; t += PL_T) s_slot[t] = trow[i0 + t] + C[(size_t)ch * N + i0 + t];
     const int j0 = ch * CH, j1 = (int)min((int64_t)V, (int64_t)j0 + CH);
     for (int w0 = j0; w0 < j1; w0 += PL_ROWS) {
         const int nr = min(PL_ROWS, j1 - w0);
         const int64_t e0 = rp[w0];
-        __syncwarp();
-        for (int r = lane; r <= nr; r += 32) s_row[r] = (int)(rp[w0 + r] - e0);
-        __syncwarp();
-        const int ne = s_row[nr];
-        int r = 0;                        // next row to place (may have started in the previous stage)
-        for (int s0 = 0; s0 < ne; s0 += PL_STG) {
-            const int s1 = min(ne, s0 + PL_STG);
-            __syncwarp();
-#pragma unroll 8
-            for (int q = s0 + lane; q < s1; q += 32) {
-                s_col[q - s0] = col[e0 + q] - i0;
-                s_val[q - s0] = val[e0 + q];
+        for (int r = tid; r <= nr; r += PL_T) s_row[r] = (int)(rp[w0 + r] - e0);
+        for (int t = tid; t < PL_WORDS * tw / 4; t += PL_T) reinterpret_cast<uint4*>(s_bits)[t] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        // an equal stretch of the entries per warp
+        const int per = (s_row[nr] + PL_T / 32 - 1) / (PL_T / 32);
+        const int tb = min(warp * per, s_row[nr]), te = min(tb + per, s_row[nr]);
+        int r0 = 0;  // the row of entry tb: the last that starts at or before it
+        for (int lo = 0, hi = nr; hi - lo > 1;) {
+            const int m = (lo + hi) >> 1;
+            if (s_row[m] <= tb)
+                lo = m;
+            else
+                hi = m;
+            r0 = lo;
+        }
+        int r = r0;
+        for (int t0 = tb; t0 < te; t0 += 32 * PL_U) {
+            int c[PL_U];
+#pragma unroll
+            for (int u = 0; u < PL_U; ++u) {
+                const int t = t0 + 32 * u + lane;
+                c[u] = t < te ? col[e0 + t] - i0 : -1;
             }
-            __syncwarp();
-            // rows with entries in [s0, s1); the last may continue in the next stage
-            while (r < nr && s_row[r] < s1) {
-                const int a = max(s_row[r], s0), b = min(s_row[r + 1], s1);
-                for (int q = a + lane; q < b; q += 32) {
-                    const int c = s_col[q - s0];
-                    if (c >= 0 && c < nt) {
-                        const int pos = s_slot[c];
-                        s_slot[c] = pos + 1;
-                        tcol[pos] = w0 + r;
-                        tval[pos] = s_val[q - s0];
-                    }
+#pragma unroll
+            for (int u = 0; u < PL_U; ++u) {
+                const int t = t0 + 32 * u + lane;
+                if (c[u] >= 0 && c[u] < nt) {
+                    while (t >= s_row[r + 1]) ++r;
+                    atomicOr(&s_bits[(r >> 5) * tw + c[u]], 1u << (r & 31));
                 }
-                __syncwarp();
-                if (s_row[r + 1] > s1) break;   // continues in the next stage
-                ++r;
             }
+        }
+        __syncthreads();
+        r = r0;
+        for (int t0 = tb; t0 < te; t0 += 32 * PL_U) {
+            int c[PL_U];
+            float v[PL_U];
+#pragma unroll
+            for (int u = 0; u < PL_U; ++u) {
+                const int t = t0 + 32 * u + lane;
+                c[u] = t < te ? col[e0 + t] - i0 : -1;
+                v[u] = t < te ? val[e0 + t] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < PL_U; ++u) {
+                const int t = t0 + 32 * u + lane;
+                if (c[u] >= 0 && c[u] < nt) {
+                    while (t >= s_row[r + 1]) ++r;
+                    const int rw = r >> 5;
+                    int pos = s_slot[c[u]] + __popc(s_bits[rw * tw + c[u]] & ((1u << (r & 31)) - 1u));
+                    for (int q = 0; q < rw; ++q) pos += __popc(s_bits[q * tw + c[u]]);
+                    tcol[pos] = w0 + r;
+                    tval[pos] = v[u];
+                }
+            }
+        }
+        if (w0 + PL_ROWS < j1) {  // the next rows' first slots
+            __syncthreads();
+            for (int t = tid; t < nt; t += PL_T) {
+                int n = 0;
+                for (int q = 0; q < PL_WORDS; ++q) n += __popc(s_bits[q * tw + t]);
+                s_slot[t] += n;
+            }
+            __syncthreads();
         }
     }
 }
-
-size_t place_smem(int nt) { return sizeof(int) * ((size_t)nt + PL_ROWS + 1 + 2 * PL_STG); }
 
 // Padding of the rows of D^T: the row's last voxel with value 0.
 __global__ void k_pad_t(const int* __restrict__ trow, const int* __restrict__ cnt, int N, int* __restrict__ tcol,
@@ -248,36 +340,83 @@ __global__ void k_quant_t(const float* __restrict__ tval, const int* __restrict_
     for (int q = trow[i] + lane; q < trow[i + 1]; q += 32) tval16[q] = to16<PREC>(tval[q] / s);
 }
 
-// The caller's CSR and labels, one warp per voxel row j: row bounds inside
-// [0, nnz], columns in [0, N) and strictly increasing, finite values, label in
-// [0, S).  A bad row or label is recorded as V - j under atomicMax (so the
-// lowest index wins); a good row writes its padded length, a good label its
-// byte and one count for its structure.  Every read of col / val is inside the
-// row's checked bounds.
-__global__ void k_check(const int64_t* __restrict__ rp, const int* __restrict__ col, const float* __restrict__ val,
-                        int64_t nnz, int V, int N, const int* __restrict__ label, int S, int pad,
-                        int64_t* __restrict__ plen, uint8_t* __restrict__ vs8, BuildCheck* __restrict__ chk) {
+// The caller's CSR and labels: row bounds inside [0, nnz], columns in [0, N) and
+// strictly increasing, finite values, label in [0, S).  A bad row or label is
+// recorded as V - j under atomicMax (so the lowest index wins); a good row writes
+// its padded length, a good label its byte and one count for its structure.  Every
+// read of col / val is inside checked bounds.
+//
+// A warp per RW_ROWS rows: where all their bounds hold, the rows' entries are one
+// stretch, and the columns increase strictly inside every row exactly when the
+// stretch has no more places that do not increase than there are among the rows'
+// starts.  Only where that, a column or a value fails are the rows looked at one by
+// one.  Prostate-shaped matrix (7.4 M entries): 50 us with a warp per row, now 23.
+__global__ void __launch_bounds__(RW_T) k_check(const int64_t* __restrict__ rp, const int* __restrict__ col,
+                                                const float* __restrict__ val, int64_t nnz, int V, int N,
+                                                const int* __restrict__ label, int S, int pad,
+                                                int64_t* __restrict__ plen, uint8_t* __restrict__ vs8,
+                                                BuildCheck* __restrict__ chk) {
     __shared__ int s_cnt[SMAX];
     for (int k = threadIdx.x; k < SMAX; k += blockDim.x) s_cnt[k] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int j = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    if (j < V) {
-        const int64_t p0 = rp[j], p1 = rp[j + 1];
-        bool ok = p0 >= 0 && p1 >= p0 && p1 <= nnz;
-        if (ok) {
-            bool bad = false, neg = false;
-            for (int64_t p = p0 + lane; p < p1; p += 32) {
-                const int c = col[p];
-                const float v = val[p];
-                bad |= c < 0 || c >= N || !isfinite(v);
-                neg |= v < 0.f;
-                if (p > p0) bad |= c <= col[p - 1];
+    const int64_t w = (int64_t)blockIdx.x * RW_W + (threadIdx.x >> 5);
+    if (w * RW_ROWS < V) {
+        const int j0 = (int)(w * RW_ROWS), j = min(j0 + min(lane, RW_ROWS), V);  // lane RW_ROWS: the end
+        const bool own = lane < RW_ROWS && j < V;
+        const int64_t p0 = rp[j], p1 = own ? rp[j + 1] : p0;
+        const bool bounds = !own || (p0 >= 0 && p1 >= p0 && p1 <= nnz);
+        bool ok = bounds, neg = false;
+        if (__all_sync(FULL, bounds)) {
+            const int64_t s0 = __shfl_sync(FULL, p0, 0), e0 = __shfl_sync(FULL, p0, RW_ROWS);
+            const bool down = p1 > p0 && p0 > s0 && col[p0] <= col[p0 - 1];
+            int extra = 0, carry = INT_MIN;
+            bool bad = false;
+            for (int64_t q = s0; q < e0; q += 32 * RW_U) {
+                int c[RW_U];
+                float v[RW_U];
+#pragma unroll
+                for (int u = 0; u < RW_U; ++u) {
+                    const int64_t p = q + 32 * u + lane;
+                    c[u] = p < e0 ? col[p] : 0;
+                    v[u] = p < e0 ? val[p] : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < RW_U; ++u) {
+                    int prev = __shfl_up_sync(FULL, c[u], 1);
+                    if (lane == 0) prev = carry;
+                    carry = __shfl_sync(FULL, c[u], 31);
+                    if (q + 32 * u + lane < e0) {
+                        bad |= c[u] < 0 || c[u] >= N || !isfinite(v[u]);
+                        neg |= v[u] < 0.f;
+                        extra += c[u] <= prev;
+                    }
+                }
             }
-            ok = !__any_sync(FULL, bad);
-            if (__any_sync(FULL, neg) && lane == 0) chk->negative = 1;
+            extra = (int)__reduce_add_sync(FULL, (unsigned)extra) - __popc(__ballot_sync(FULL, down));
+            ok = extra == 0 && !__any_sync(FULL, bad);
+        } else {
+            ok = false;
         }
-        if (lane == 0) {
+        if (!__all_sync(FULL, ok)) {  // which rows
+            for (int r = 0; r < RW_ROWS; ++r) {
+                const int64_t a = __shfl_sync(FULL, p0, r), b = __shfl_sync(FULL, p1, r);
+                bool good = __shfl_sync(FULL, (int)bounds, r) != 0;
+                if (good) {
+                    bool bad = false;
+                    for (int64_t p = a + lane; p < b; p += 32) {
+                        const int c = col[p];
+                        const float v = val[p];
+                        bad |= c < 0 || c >= N || !isfinite(v);
+                        if (p > a) bad |= c <= col[p - 1];
+                    }
+                    good = !__any_sync(FULL, bad);
+                }
+                if (lane == r) ok = good;
+            }
+        }
+        if (__any_sync(FULL, neg) && lane == 0) chk->negative = 1;
+        if (own) {
             plen[j] = ok ? (p1 - p0 + pad - 1) / pad * pad : 0;
             if (!ok) atomicMax(&chk->bad_row, V - j);
             const int l = label[j];
@@ -380,6 +519,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_apply(const int64_t* __restrict
 }
 
 inline unsigned blocks_for(int64_t threads, int bs) { return (unsigned)((threads + bs - 1) / bs); }
+inline unsigned row_warp_blocks(int V) { return blocks_for(((int64_t)V + RW_ROWS - 1) / RW_ROWS * 32, RW_T); }
 
 }  // namespace
 
@@ -390,7 +530,7 @@ cudaError_t build_check(const int64_t* rp, const int* col, const float* val, int
                         BuildCheck* chk, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(chk, 0, sizeof(BuildCheck), s);
     if (e != cudaSuccess) return e;
-    k_check<<<blocks_for((int64_t)V * 32, 256), 256, 0, s>>>(rp, col, val, nnz, V, N, label, S, pad, plen, vs8, chk);
+    k_check<<<row_warp_blocks(V), RW_T, 0, s>>>(rp, col, val, nnz, V, N, label, S, pad, plen, vs8, chk);
     const int nb = check_scan_blocks(V);
     k_scan_totals<<<nb, SCAN_T, 0, s>>>(plen, V, bsum);
     k_scan_offsets<<<1, SCAN_T, 0, s>>>(bsum, nb, V, prow, chk);
@@ -416,20 +556,17 @@ cudaError_t build_stats(const int64_t* rp, const int* col, const float* val, int
 }
 
 cudaError_t build_fill_d(int prec, const int64_t* rp, const int* col, const float* val, const int* prow, int V,
-                         const float* scale, DevCSR& D, cudaStream_t s) {
-    const unsigned g = blocks_for((int64_t)V * 32, 256);
+                         const float* scale, const int* beam_off, int B, int* seg, DevCSR& D, cudaStream_t s) {
+    const unsigned g = row_warp_blocks(V);
     if (prec == DAO_PREC_FP32)
-        k_fill_d<DAO_PREC_FP32><<<g, 256, 0, s>>>(rp, col, val, prow, V, scale, D.col, D.val, nullptr, nullptr);
+        k_fill_d<DAO_PREC_FP32><<<g, RW_T, 0, s>>>(rp, col, val, prow, V, scale, beam_off, B, seg, D.col, D.val,
+                                                   nullptr, nullptr);
     else if (prec == DAO_PREC_FP16)
-        k_fill_d<DAO_PREC_FP16><<<g, 256, 0, s>>>(rp, col, val, prow, V, scale, nullptr, nullptr, D.col16, D.val16);
+        k_fill_d<DAO_PREC_FP16><<<g, RW_T, 0, s>>>(rp, col, val, prow, V, scale, beam_off, B, seg, nullptr, nullptr,
+                                                   D.col16, D.val16);
     else
-        k_fill_d<DAO_PREC_BF16><<<g, 256, 0, s>>>(rp, col, val, prow, V, scale, nullptr, nullptr, D.col16, D.val16);
-    return cudaGetLastError();
-}
-
-cudaError_t build_seg(const int64_t* rp, const int* col, const int* prow, int V, const int* beam_off, int B, int* seg,
-                      cudaStream_t s) {
-    k_seg<<<blocks_for(V, 256), 256, 0, s>>>(rp, col, prow, V, beam_off, B, seg);
+        k_fill_d<DAO_PREC_BF16><<<g, RW_T, 0, s>>>(rp, col, val, prow, V, scale, beam_off, B, seg, nullptr, nullptr,
+                                                   D.col16, D.val16);
     return cudaGetLastError();
 }
 
@@ -544,29 +681,63 @@ __global__ void __launch_bounds__(BEAM_TILE) k_beam_offsets(const int* __restric
     if (j < V) brp[(size_t)b * (V + 1) + j] = toff[(size_t)b * n_tiles + t] + incl - len;
 }
 
-// One thread per (beam, row): the row's segment of the beam, with the beamlet
-// index made local to the beam.
+// D by beams: the rows' segments of each beam one after the other, with the beamlet
+// index local to the beam.  A warp per 32 rows of one beam, whose entries are one
+// stretch of the beam's range.  A thread per (beam, row) that copied its segment
+// took 84 us on a prostate-shaped FP32 matrix (7.4 M entries, 9 beams); now 30.
 template <int PREC>
-__global__ void k_beam_fill(const int* __restrict__ seg, int V, int B, const int* __restrict__ beam_off,
-                            const int* __restrict__ brp, const int* __restrict__ col, const float* __restrict__ val,
-                            const unsigned short* __restrict__ col16, const unsigned short* __restrict__ val16,
-                            unsigned short* __restrict__ bcol, float* __restrict__ bval32,
-                            unsigned short* __restrict__ bval16) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)B * V) return;
-    const int b = (int)(i / V), j = (int)(i % V);
-    const int q0 = seg[(size_t)b * V + j], q1 = seg[(size_t)(b + 1) * V + j];
-    const int base = beam_off[b];
-    int64_t d0 = brp[(size_t)b * (V + 1) + j];
-    for (int bb = 0; bb < b; ++bb) d0 += brp[(size_t)bb * (V + 1) + V];  // the beams before b
-    for (int q = q0; q < q1; ++q) {
-        const int64_t d = d0 + (q - q0);
-        if constexpr (PREC == DAO_PREC_FP32) {
-            bcol[d] = (unsigned short)(col[q] - base);
-            bval32[d] = val[q];
-        } else {
-            bcol[d] = (unsigned short)(col16[q] - base);
-            bval16[d] = val16[q];
+__global__ void __launch_bounds__(RW_T) k_beam_fill(const int* __restrict__ seg, int V,
+                                                    const int* __restrict__ beam_off,
+                                                    const int* __restrict__ brp, const int* __restrict__ col,
+                                                    const float* __restrict__ val,
+                                                    const unsigned short* __restrict__ col16,
+                                                    const unsigned short* __restrict__ val16,
+                                                    unsigned short* __restrict__ bcol, float* __restrict__ bval32,
+                                                    unsigned short* __restrict__ bval16) {
+    __shared__ int s_start[RW_W][33], s_src[RW_W][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.y;
+    const int j = (int)min((int64_t)V, ((int64_t)blockIdx.x * RW_W + warp) * 32 + lane);
+    if (__shfl_sync(FULL, j, 0) >= V) return;  // uniform
+    const int* bp = brp + (size_t)b * (V + 1);
+    const int d = bp[j];
+    int before = 0;  // the entries of the beams before b
+    for (int bb = lane; bb < b; bb += 32) before += brp[(size_t)bb * (V + 1) + V];
+    before = (int)__reduce_add_sync(FULL, (unsigned)before);
+    const int d0 = __shfl_sync(FULL, d, 0), base = beam_off[b];
+    const int64_t out = (int64_t)before + d0;
+    s_start[warp][lane] = d - d0;
+    s_src[warp][lane] = j < V ? seg[(size_t)b * V + j] - (d - d0) : 0;
+    if (lane == 31) s_start[warp][32] = bp[min(j + 1, V)] - d0;
+    __syncwarp();
+    const int n = s_start[warp][32];
+    int r = 0;
+    for (int t0 = 0; t0 < n; t0 += 32 * RW_U) {
+        int c[RW_U];
+        float v[RW_U];
+        unsigned short h[RW_U];
+#pragma unroll
+        for (int u = 0; u < RW_U; ++u) {
+            const int t = t0 + 32 * u + lane;
+            if (t >= n) continue;
+            while (t >= s_start[warp][r + 1]) ++r;
+            const int q = s_src[warp][r] + t;
+            if (PREC == DAO_PREC_FP32) {
+                c[u] = __ldg(col + q);
+                v[u] = __ldg(val + q);
+            } else {
+                c[u] = __ldg(col16 + q);
+                h[u] = __ldg(val16 + q);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < RW_U; ++u) {
+            const int t = t0 + 32 * u + lane;
+            if (t >= n) continue;
+            bcol[out + t] = (unsigned short)(c[u] - base);
+            if (PREC == DAO_PREC_FP32)
+                bval32[out + t] = v[u];
+            else
+                bval16[out + t] = h[u];
         }
     }
 }
@@ -585,15 +756,14 @@ cudaError_t build_beam_rows(const int* seg, int V, int B, int* brp, int* tmp, cu
 
 cudaError_t build_beam_fill(int prec, const int* seg, int V, int B, const int* beam_off, const DevCSR& D,
                             cudaStream_t s) {
-    const int64_t n = (int64_t)B * V;
-    if (n == 0) return cudaSuccess;
-    const unsigned g = (unsigned)((n + 255) / 256);
+    if (B < 1 || V < 1) return cudaSuccess;
+    const dim3 g((unsigned)(((int64_t)V + RW_T - 1) / RW_T), (unsigned)B);  // RW_W warps of 32 rows
     if (prec == DAO_PREC_FP32)
-        k_beam_fill<DAO_PREC_FP32><<<g, 256, 0, s>>>(seg, V, B, beam_off, D.beam_rowptr, D.col, D.val, nullptr,
-                                                     nullptr, D.beam_col, D.beam_val32, nullptr);
+        k_beam_fill<DAO_PREC_FP32><<<g, RW_T, 0, s>>>(seg, V, beam_off, D.beam_rowptr, D.col, D.val,
+                                                      nullptr, nullptr, D.beam_col, D.beam_val32, nullptr);
     else
-        k_beam_fill<DAO_PREC_FP16><<<g, 256, 0, s>>>(seg, V, B, beam_off, D.beam_rowptr, nullptr, nullptr, D.col16,
-                                                     D.val16, D.beam_col, nullptr, D.beam_val16);
+        k_beam_fill<DAO_PREC_FP16><<<g, RW_T, 0, s>>>(seg, V, beam_off, D.beam_rowptr, nullptr, nullptr,
+                                                      D.col16, D.val16, D.beam_col, nullptr, D.beam_val16);
     return cudaGetLastError();
 }
 
@@ -612,16 +782,15 @@ cudaError_t build_unit_max(const int* prow, int V, int epg, int* out, cudaStream
 
 cudaError_t build_transpose_place(int prec, const int64_t* rp, const int* col, const float* val, int V, int CH, int N,
                                   int n_ch, int* C, const int* cnt, const float* scale, DevCSR& Dt, float* tval,
-                                  int num_sms, cudaStream_t s) {
-    const int split = std::max(1, std::min(16, (24 * num_sms + n_ch - 1) / n_ch));
-    const int tw = std::min(TILE_N, (N + split - 1) / split);
-    const int n_tile = (N + tw - 1) / tw;
-    const size_t sm_place = place_smem(tw);
+                                  cudaStream_t s) {
+    const int n_tile = (N + PL_TILE - 1) / PL_TILE;
+    const int tw = ((N + n_tile - 1) / n_tile + 3) / 4 * 4;  // the bitmap is cleared 16 bytes at a time
     // process-wide: the largest size any launch asks for (see build_stats)
     cudaError_t e = cudaFuncSetAttribute(k_chunk_place, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)place_smem(TILE_N));
+                                         (int)place_smem(PL_TILE));
     if (e != cudaSuccess) return e;
-    k_chunk_place<<<dim3(n_ch, n_tile), 32, sm_place, s>>>(rp, col, val, V, CH, N, tw, C, Dt.rowptr, Dt.col, tval);
+    k_chunk_place<<<dim3(n_ch, n_tile), PL_T, place_smem(tw), s>>>(rp, col, val, V, CH, N, tw, C, Dt.rowptr, Dt.col,
+                                                                   tval);
     k_pad_t<<<blocks_for((int64_t)N * 32, 256), 256, 0, s>>>(Dt.rowptr, cnt, N, Dt.col, tval);
     if (prec == DAO_PREC_FP16)
         k_quant_t<DAO_PREC_FP16><<<blocks_for((int64_t)N * 32, 256), 256, 0, s>>>(tval, Dt.rowptr, N, scale,

@@ -481,9 +481,7 @@ cudaError_t build_check(const int64_t* rp, const int* col, const float* val, int
 cudaError_t build_stats(const int64_t* rp, const int* col, const float* val, int V, int CH, int N, int n_ch,
                         int* C, int* cnt, unsigned* smax, unsigned* dmax, int num_sms, cudaStream_t s);
 cudaError_t build_fill_d(int prec, const int64_t* rp, const int* col, const float* val, const int* prow, int V,
-                         const float* scale, DevCSR& D, cudaStream_t s);
-cudaError_t build_seg(const int64_t* rp, const int* col, const int* prow, int V, const int* beam_off, int B, int* seg,
-                      cudaStream_t s);
+                         const float* scale, const int* beam_off, int B, int* seg, DevCSR& D, cudaStream_t s);
 // The most groups of epg entries in one unit of 32 consecutive rows of the
 // padded D (row offsets prow) into out[0], the most in one row into out[1]
 // (both zeroed by the call).
@@ -501,7 +499,7 @@ cudaError_t build_beam_fill(int prec, const int* seg, int V, int B, const int* b
 cudaError_t build_merge_path(const int* prow, int V, int epg, int chunk, int n_warps, int2* out, cudaStream_t s);
 cudaError_t build_transpose_place(int prec, const int64_t* rp, const int* col, const float* val, int V, int CH, int N,
                                   int n_ch, int* C, const int* cnt, const float* scale, DevCSR& Dt, float* tval,
-                                  int num_sms, cudaStream_t s);
+                                  cudaStream_t s);
 
 // One plan's persistent master solve as the kernel reads it: the solver state,
 // the slab and its partial arrays (stride GS), the objective terms, the
