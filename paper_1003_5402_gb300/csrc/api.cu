@@ -883,7 +883,6 @@ dao_status append_apertures(dao_ctx* c, int n, const int32_t* beams, const int32
     }
     c->ap_beam_h.insert(c->ap_beam_h.end(), beams, beams + n);
     c->ap_lr_h.resize((size_t)(K0 + n) * stride, 0);
-    std::vector<ColumnList> list(c->B, ColumnList{});
     for (int i = 0; i < n; ++i) {
         const int32_t* lr = leaf_lr + (size_t)i * stride;
         for (int r = 0; r < c->rows[beams[i]]; ++r) {
@@ -896,19 +895,19 @@ dao_status append_apertures(dao_ctx* c, int n, const int32_t* beams, const int32
     DAO_CU(cudaMemcpyAsync(c->ap_lr + (size_t)K0 * stride, &c->ap_lr_h[(size_t)K0 * stride],
                            sizeof(int) * (size_t)n * stride, cudaMemcpyHostToDevice, c->stream));
     c->prof_begin(DAO_KC_COLUMN);
-    auto flush = [&](int b) -> cudaError_t {
-        const cudaError_t e = launch_columns(c->D, b, c->beam_off[b], c->rows[b], c->cols[b], list[b], c->ap_lr,
-                                             stride, c->slab, c->ld, c->num_sms, c->stream, &c->launches_i);
-        list[b].n = 0;
-        return e;
-    };
+    ColumnLists lists;
+    lists.n = 0;
+    std::vector<int> open(c->B, -1);  // the beam's list that still has room
     for (int i = 0; i < n; ++i) {
-        ColumnList& l = list[beams[i]];
+        const int b = beams[i];
+        if (open[b] < 0 || lists.list[open[b]].n == COLUMNS_MAX) {
+            open[b] = lists.n++;
+            lists.list[open[b]] = ColumnList{b, c->beam_off[b], c->rows[b], c->cols[b], 0, {}};
+        }
+        ColumnList& l = lists.list[open[b]];
         l.k[l.n++] = K0 + i;
-        if (l.n == COLUMNS_MAX) DAO_CU(flush(beams[i]));
     }
-    for (int b = 0; b < c->B; ++b)
-        if (list[b].n > 0) DAO_CU(flush(b));
+    DAO_CU(launch_columns(c->D, lists, c->ap_lr, stride, c->slab, c->ld, c->num_sms, c->stream, &c->launches_i));
     c->prof_end();
     c->K += n;
     return DAO_OK;

@@ -242,19 +242,23 @@ cudaError_t launch_column_dev(const DevCSR& D, const int* seg, const int* ap_bea
                               const int* rows, const int* cols, int max_nb, const float* mask, float* slab, int ld,
                               const CGDev* cg, int num_sms, cudaStream_t stream, int* launches);
 
-// a4 for up to COLUMNS_MAX apertures of beam b, pool indices k[0 .. n), from the
-// device's aperture table into their slab columns, reading the beam's part of D
-// once.  columns_available: a4 runs on D by beams and the largest beam's table
+// a4 for lists of up to COLUMNS_MAX apertures of one beam each, pool indices
+// k[0 .. n), from the device's aperture table into their slab columns, reading the
+// beam's part of D once per list; all lists in one launch.  columns_available: a4 runs on D by beams and the largest beam's table
 // (max_nb beamlets) fits the default shared memory.
 bool columns_available(const DevCSR& D, int max_nb);
 constexpr int COLUMNS_MAX = 8;
 struct ColumnList {
+    int beam, base, rows, cols;  // the beam, its first beamlet, its MLC rows and columns
     int n;
     int k[COLUMNS_MAX];
 };
-cudaError_t launch_columns(const DevCSR& D, int b, int base, int rows, int cols, const ColumnList& list,
-                           const int* ap_lr, int lr_stride, float* slab, int ld, int num_sms, cudaStream_t stream,
-                           int* launches);
+struct ColumnLists {
+    int n;
+    ColumnList list[KMAX];
+};
+cudaError_t launch_columns(const DevCSR& D, const ColumnLists& lists, const int* ap_lr, int lr_stride, float* slab,
+                           int ld, int num_sms, cudaStream_t stream, int* launches);
 
 // x_i = sum_{k in K_i} y_k (Eq. 7) from the aperture table.
 cudaError_t launch_fluence(const int* ap_beam, const int* ap_lr, int lr_stride, const double* y, int K,

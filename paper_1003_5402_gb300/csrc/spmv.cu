@@ -397,24 +397,25 @@ __global__ void __launch_bounds__(256) k_column_beam(const int* __restrict__ brp
                               smask, out, stride, (int)(blockIdx.x * blockDim.x), (int)(gridDim.x * blockDim.x));
 }
 
-// a4 for several apertures of one beam: one pass over the beam's part of D by
+// a4 for several apertures of one beam (a list per blockIdx.y): one pass over the beam's part of D by
 // beams, a bit per aperture and beamlet in shared memory; each column's sum takes
 // the open entries in order, the arithmetic of column_beam_body (a closed
 // entry's product is 0 there).  An imported pool of 40 apertures on the
 // H&N-shaped matrix took 40 launches of 8.8 us with a mask upload and a
-// synchronisation each.
+// synchronisation each; with a launch per list (5, of up to 17 us, each too small
+// to fill the chip) the import took 659 us, with one launch 627.
 template <bool W16, bool BF>
 __global__ void __launch_bounds__(256) k_columns_beam(const int* __restrict__ brp_all,
                                                       const unsigned short* __restrict__ bcol,
                                                       const float* __restrict__ bval32,
-                                                      const unsigned short* __restrict__ bval16, int V, int b,
-                                                      int base, int rows, int cols,
-                                                      const __grid_constant__ ColumnList list,
+                                                      const unsigned short* __restrict__ bval16, int V,
+                                                      const __grid_constant__ ColumnLists lists,
                                                       const int* __restrict__ ap_lr, int lr_stride,
                                                       const float* __restrict__ scale, float* __restrict__ slab,
                                                       int ld) {
     extern __shared__ float2 s_open[];  // per beamlet: the scale (1 for FP32 values), the apertures' bits
-    const int nb = rows * cols;
+    const ColumnList& list = lists.list[blockIdx.y];
+    const int b = list.beam, base = list.base, cols = list.cols, nb = list.rows * cols;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) {
         const int r = i / cols, c = i % cols;
         unsigned m = 0u;
@@ -1347,25 +1348,23 @@ bool columns_available(const DevCSR& D, int max_nb) {
     return column_by_beams(D) && (size_t)max_nb * sizeof(float2) <= 48 * 1024;
 }
 
-cudaError_t launch_columns(const DevCSR& D, int b, int base, int rows, int cols, const ColumnList& list,
-                           const int* ap_lr, int lr_stride, float* slab, int ld, int num_sms, cudaStream_t stream,
-                           int* launches) {
-    if (!columns_available(D, rows * cols)) return cudaErrorNotSupported;
-    if (D.n_rows == 0 || list.n == 0) return cudaSuccess;
-    const size_t sm = (size_t)rows * cols * sizeof(float2);
-    const int grid = std::min(num_sms * 8, (D.n_rows + 255) / 256);
+cudaError_t launch_columns(const DevCSR& D, const ColumnLists& lists, const int* ap_lr, int lr_stride, float* slab,
+                           int ld, int num_sms, cudaStream_t stream, int* launches) {
+    int nb = 0;
+    for (int g = 0; g < lists.n; ++g) nb = std::max(nb, lists.list[g].rows * lists.list[g].cols);
+    if (!columns_available(D, nb)) return cudaErrorNotSupported;
+    if (D.n_rows == 0 || lists.n == 0) return cudaSuccess;
+    const size_t sm = (size_t)nb * sizeof(float2);
+    const dim3 grid((unsigned)std::min(num_sms * 8, (D.n_rows + 255) / 256), (unsigned)lists.n);
     if (D.prec == DAO_PREC_FP16)
         k_columns_beam<true, false><<<grid, 256, sm, stream>>>(D.beam_rowptr, D.beam_col, nullptr, D.beam_val16,
-                                                                D.n_rows, b, base, rows, cols, list, ap_lr, lr_stride,
-                                                                D.scale, slab, ld);
+                                                                D.n_rows, lists, ap_lr, lr_stride, D.scale, slab, ld);
     else if (D.prec == DAO_PREC_BF16)
         k_columns_beam<true, true><<<grid, 256, sm, stream>>>(D.beam_rowptr, D.beam_col, nullptr, D.beam_val16,
-                                                               D.n_rows, b, base, rows, cols, list, ap_lr, lr_stride,
-                                                               D.scale, slab, ld);
+                                                               D.n_rows, lists, ap_lr, lr_stride, D.scale, slab, ld);
     else
         k_columns_beam<false, false><<<grid, 256, sm, stream>>>(D.beam_rowptr, D.beam_col, D.beam_val32, nullptr,
-                                                                 D.n_rows, b, base, rows, cols, list, ap_lr,
-                                                                 lr_stride, D.scale, slab, ld);
+                                                                 D.n_rows, lists, ap_lr, lr_stride, D.scale, slab, ld);
     ++*launches;
     return cudaGetLastError();
 }
