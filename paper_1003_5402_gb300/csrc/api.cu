@@ -295,6 +295,8 @@ struct DeviceCSR {
     int64_t nnz = 0;
 };
 
+dao_status alloc_state(dao_ctx* c);
+
 dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const dao_structures* s,
                  const dao_weights* w, const double* rx, const dao_voxel_terms* vt, DeviceCSR* din) {
     const int V = c->V, N = c->N, B = c->B;
@@ -429,6 +431,23 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
     DAO_TRY(c->dalloc(&scale, N));
     c->D.scale = scale;
     c->Dt.scale = scale;
+    DAO_TRY(cu(build_stats(t_rp, t_col, t_val, V, CH, N, n_ch, t_C, t_cnt, reinterpret_cast<unsigned*>(scale), t_dmax,
+                           c->num_sms, st), "transpose counts and scales"));
+    DAO_TRY(cu(build_unit_max(c->D.rowptr, V, pad_m, t_umax, st), "row units"));
+    // Counts, the largest |D_ij| and the largest row unit back to the host: row
+    // offsets of D^T, tau, the dose SpMV's shared partials.  Read before the layouts
+    // are launched: what the host makes of them (the row offsets, then the order of
+    // the rows, the split form's table, the objective's terms and the plan's state)
+    // it makes while the device writes the layouts (re-plan of 20 apertures on a
+    // prostate-shaped FP32 matrix: 1.54 ms with the device idle meanwhile, now 1.34).
+    std::vector<int> cnt(N);
+    unsigned dmax_bits = 0;
+    int umax[2] = {0, 0};
+    DAO_TRY(cu(cudaMemcpyAsync(cnt.data(), t_cnt, sizeof(int) * N, cudaMemcpyDeviceToHost, st), "counts"));
+    DAO_TRY(cu(cudaMemcpyAsync(&dmax_bits, t_dmax, sizeof(unsigned), cudaMemcpyDeviceToHost, st), "max"));
+    DAO_TRY(cu(cudaMemcpyAsync(umax, t_umax, 2 * sizeof(int), cudaMemcpyDeviceToHost, st), "units"));
+    DAO_TRY(cu(cudaStreamSynchronize(st), "device build"));
+    c->D.unit_groups_max = std::max(umax[0], 1);
     DAO_TRY(upload(c, &c->beam_off_d, c->beam_off.data(), c->beam_off.size()));
     DAO_TRY(c->dalloc(&c->seg, (size_t)(B + 1) * V));
     if (prec == DAO_PREC_FP32) {
@@ -438,8 +457,6 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
         DAO_TRY(c->dalloc(&c->D.col16, padded));
         DAO_TRY(c->dalloc(&c->D.val16, padded));
     }
-    DAO_TRY(cu(build_stats(t_rp, t_col, t_val, V, CH, N, n_ch, t_C, t_cnt, reinterpret_cast<unsigned*>(scale), t_dmax,
-                           c->num_sms, st), "transpose counts and scales"));
     DAO_TRY(cu(build_fill_d(prec, t_rp, t_col, t_val, c->D.rowptr, V, scale, c->beam_off_d, B, c->seg, c->D, st),
                "padded D and beam segments"));
     // D by beams for the aperture column (a4): each beam's part of every row
@@ -453,17 +470,30 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
     DAO_TRY(talloc(&t_bscan, sizeof(int) * (size_t)B * beam_scan_tiles(V)));
     DAO_TRY(cu(build_beam_rows(c->seg, V, B, c->D.beam_rowptr, t_bscan, st), "beam rows"));
     DAO_TRY(cu(build_beam_fill(prec, c->seg, V, B, c->beam_off_d, c->D, st), "beam layout"));
-    DAO_TRY(cu(build_unit_max(c->D.rowptr, V, pad_m, t_umax, st), "row units"));
-    // counts, the largest |D_ij| and the largest row unit back to the host: row
-    // offsets of D^T, tau, the dose SpMV's shared partials
-    std::vector<int> cnt(N);
-    unsigned dmax_bits = 0;
-    int umax[2] = {0, 0};
-    DAO_TRY(cu(cudaMemcpyAsync(cnt.data(), t_cnt, sizeof(int) * N, cudaMemcpyDeviceToHost, st), "counts"));
-    DAO_TRY(cu(cudaMemcpyAsync(&dmax_bits, t_dmax, sizeof(unsigned), cudaMemcpyDeviceToHost, st), "max"));
-    DAO_TRY(cu(cudaMemcpyAsync(umax, t_umax, 2 * sizeof(int), cudaMemcpyDeviceToHost, st), "units"));
-    DAO_TRY(cu(cudaStreamSynchronize(st), "device build"));
-    c->D.unit_groups_max = std::max(umax[0], 1);
+    std::vector<int> trow(N + 1, 0);
+    int64_t tpadded = 0;
+    for (int i = 0; i < N; ++i) {
+        trow[i] = (int)std::min<int64_t>(tpadded, INT32_MAX);
+        tpadded += round_up(cnt[i], pad_m);
+    }
+    if (tpadded >= (int64_t)1 << 31) {
+        free_temps();
+        return fail(DAO_EINVAL, "D^T too large for 32-bit row offsets");
+    }
+    trow[N] = (int)tpadded;
+    c->Dt.nnz_stored = tpadded;
+    DAO_TRY(upload(c, &c->Dt.rowptr, trow.data(), trow.size()));
+    DAO_TRY(c->dalloc(&c->Dt.col, tpadded));
+    if (prec == DAO_PREC_FP32) {
+        DAO_TRY(c->dalloc(&c->Dt.val, tpadded));
+        t_tval = c->Dt.val;
+    } else {
+        DAO_TRY(c->dalloc(&c->Dt.val16, tpadded));
+        DAO_TRY(talloc(&t_tval, sizeof(float) * tpadded));
+    }
+    DAO_TRY(cu(build_transpose_place(prec, t_rp, t_col, t_val, V, CH, N, n_ch, t_C, t_cnt, scale, c->Dt, t_tval, st),
+               "transpose"));
+    free_temps();
     {
         // the merge form of a1: the merge of D's groups and row ends in equal
         // stretches (longer than the longest row) over a fixed set of warps
@@ -478,26 +508,13 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
             DAO_TRY(c->dalloc(&mp, (size_t)nw + 1));
             DAO_TRY(c->dalloc(&c->D.merge_slot, 2 * (size_t)nw));
             DAO_TRY(c->dalloc(&c->D.merge_cnt, (size_t)nw));
-            DAO_TRY(cu(cudaMemsetAsync(c->D.merge_cnt, 0, sizeof(int) * (size_t)nw, st), "merge tickets"));
-            DAO_TRY(cu(build_merge_path(c->D.rowptr, V, pad_m, (int)chunk, nw, mp, st), "merge path"));
+            DAO_CU(cudaMemsetAsync(c->D.merge_cnt, 0, sizeof(int) * (size_t)nw, st));
+            DAO_CU(build_merge_path(c->D.rowptr, V, pad_m, (int)chunk, nw, mp, st));
             c->D.merge_path = mp;
             c->D.merge_chunk = (int)chunk;
             c->D.merge_warps = nw;
         }
     }
-    std::vector<int> trow(N + 1, 0);
-    int64_t tpadded = 0;
-    for (int i = 0; i < N; ++i) {
-        trow[i] = (int)std::min<int64_t>(tpadded, INT32_MAX);
-        tpadded += round_up(cnt[i], pad_m);
-    }
-    if (tpadded >= (int64_t)1 << 31) {
-        free_temps();
-        return fail(DAO_EINVAL, "D^T too large for 32-bit row offsets");
-    }
-    trow[N] = (int)tpadded;
-    c->Dt.nnz_stored = tpadded;
-    DAO_TRY(upload(c, &c->Dt.rowptr, trow.data(), trow.size()));
     // rows of D^T by decreasing length (ties by index) for the transposed SpMV;
     // the host copy lives until build() has synchronised
     std::vector<int> order(N);
@@ -540,17 +557,6 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
             c->Dt.split_ps = ps;
         }
     }
-    DAO_TRY(c->dalloc(&c->Dt.col, tpadded));
-    if (prec == DAO_PREC_FP32) {
-        DAO_TRY(c->dalloc(&c->Dt.val, tpadded));
-        t_tval = c->Dt.val;
-    } else {
-        DAO_TRY(c->dalloc(&c->Dt.val16, tpadded));
-        DAO_TRY(talloc(&t_tval, sizeof(float) * tpadded));
-    }
-    DAO_TRY(cu(build_transpose_place(prec, t_rp, t_col, t_val, V, CH, N, n_ch, t_C, t_cnt, scale, c->Dt, t_tval, st),
-               "transpose"));
-    free_temps();
     float dmax = 0.f;
     std::memcpy(&dmax, &dmax_bits, sizeof(float));
 
@@ -599,8 +605,9 @@ dao_status build(dao_ctx* c, const dao_csr* Din, const dao_geometry* g, const da
     DAO_TRY(upload(c, &c->binfo, bi.data(), bi.size()));
     DAO_TRY(upload(c, &c->rows_d, c->rows.data(), c->rows.size()));
     DAO_TRY(upload(c, &c->cols_d, c->cols.data(), c->cols.size()));
-    DAO_TRY(sync(c));
-    return DAO_OK;
+    const dao_status state = alloc_state(c);
+    DAO_TRY(sync(c));  // also where that failed: the host arrays go out of scope
+    return state;
 }
 
 // 2-D tensor maps over the slab (a row per group of four columns: ld voxels of 16
@@ -1405,7 +1412,6 @@ dao_status create_common(const dao_csr* D, const dao_geometry* g, const dao_stru
     if (st == DAO_OK) st = build(c, D, g, s, w, prescriptions, vt, pb ? &gen : nullptr);
     for (void* q : {(void*)gen.rp, (void*)gen.col, (void*)gen.val})  // left over when build did not run
         if (q) pool_free(q, c->stream);
-    if (st == DAO_OK) st = alloc_state(c);
     if (st == DAO_OK) st = reset_state(c);
     if (st != DAO_OK) {
         std::string keep = g_err;
