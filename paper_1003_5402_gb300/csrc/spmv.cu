@@ -558,8 +558,9 @@ __global__ void __launch_bounds__(256) k_dose16(const int* __restrict__ rowptr, 
 }
 
 // ---- a1 in units of 32 voxel rows ------------------------------------------
-// One warp per unit of 32 consecutive rows (grid-stride over the units, every
-// block resident): the unit's entries are one contiguous range of groups (8
+// One warp per unit of 32 consecutive rows (SPREAD: of spread_rows, so that few rows
+// still reach every warp, see dose_units; grid-stride over the units, every block
+// resident): the unit's entries are one contiguous range of groups (8
 // entries of 16-bit storage, 4 of FP32), which the lanes request together,
 // lane l the groups l, l + 32, ..., up to UB per lane at a time, so that the
 // whole unit is in flight at once and every request is a full 512-byte
@@ -595,12 +596,12 @@ __device__ __forceinline__ float group_dot(const uint4 c, const uint4 v, const f
     return p;
 }
 
-template <bool L16, bool BF>
+template <bool L16, bool BF, bool SPREAD>
 __global__ void __launch_bounds__(UNIT_THREADS, 2) k_dose_units(
     const int* __restrict__ rowptr, const uint4* __restrict__ colg, const uint4* __restrict__ valg, int V,
     const float* __restrict__ x, const float* __restrict__ scale, int N, const uint8_t* __restrict__ vstruct,
     const StructTermsS* __restrict__ ts, int S, float* __restrict__ z, float* __restrict__ grad,
-    double* F_part, int part_cap, unsigned* ticket, double* F_out) {
+    double* F_part, int part_cap, int spread_rows, unsigned* ticket, double* F_out) {
     constexpr int EPG = L16 ? 8 : 4;  // entries per group (one 16-byte load of columns and of values)
     constexpr int UB = 4;             // groups per lane in flight
     constexpr int NW = UNIT_THREADS / 32;
@@ -610,17 +611,18 @@ __global__ void __launch_bounds__(UNIT_THREADS, 2) k_dose_units(
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     float* sx = s_dyn_units;
     float* spart = s_dyn_units + ((N + 3) & ~3) + wib * part_cap;
-    const int n_units = (V + UNIT_ROWS - 1) / UNIT_ROWS;
+    const int ur = SPREAD ? spread_rows : UNIT_ROWS;
+    const int n_units = (V + ur - 1) / ur;
     const int W = gridDim.x * NW;
     int u = blockIdx.x * NW + wib;
     // this unit's row offsets and labels first, so that they are in flight
     // while x is staged
     int rs = 0, re = 0, lab = 0;
     auto meta = [&](int uu, int& a, int& b, int& l) {
-        const int row = uu * UNIT_ROWS + lane;
+        const int row = uu * ur + lane;
         a = b = 0;
         l = 0;
-        if (uu < n_units && row < V) {
+        if (uu < n_units && lane < ur && row < V) {
             a = __ldg(rowptr + row);
             b = __ldg(rowptr + row + 1);
             if (S >= 0) l = __ldg(vstruct + row);
@@ -632,8 +634,8 @@ __global__ void __launch_bounds__(UNIT_THREADS, 2) k_dose_units(
     __syncthreads();
     float facc = 0.f;
     for (; u < n_units; u += W) {
-        const int row0 = u * UNIT_ROWS;
-        const int nrow = min(UNIT_ROWS, V - row0);
+        const int row0 = u * ur;
+        const int nrow = min(ur, V - row0);
         const int e0 = __shfl_sync(FULL, rs, 0);
         const int e1 = __shfl_sync(FULL, re, nrow - 1);
         int rs_n, re_n, lab_n;
@@ -1026,18 +1028,27 @@ cudaError_t dose_units(const DevCSR& D, const float* x, const uint8_t* vstruct, 
                        cudaStream_t stream) {
     const size_t smem = units_smem(D.n_cols, D.unit_groups_max);
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dose_units<L16, BF>, UNIT_THREADS, smem) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dose_units<L16, BF, false>, UNIT_THREADS, smem) !=
             cudaSuccess ||
         occ < 1) {
         cudaGetLastError();
         occ = 1;
     }
     grid = std::min(grid, occ * num_sms);
+    // Where the rows come to 16 or fewer per warp, units of that many (at least 4: a
+    // unit's entries then still fill one request): k_dose on 19,200 rows, 4 a warp
+    // instead of 32 for one warp in eight, 25.3 -> 23.6 us.  On more rows units of 32: an even
+    // split of 174,000 rows (18 + 18 a warp instead of 32 + 4) gained nothing, and
+    // a variable unit cost 34.0 -> 34.8 us on 304,184.
+    const int warps = grid * (UNIT_THREADS / 32);
+    const int per = std::max(4, (D.n_rows + warps - 1) / warps);
+    const bool spread = per <= UNIT_ROWS / 2;
     const void* colp = L16 ? static_cast<const void*>(D.col16) : static_cast<const void*>(D.col);
     const void* valp = L16 ? static_cast<const void*>(D.val16) : static_cast<const void*>(D.val);
-    k_dose_units<L16, BF><<<grid, UNIT_THREADS, smem, stream>>>(
+    auto kernel = spread ? k_dose_units<L16, BF, true> : k_dose_units<L16, BF, false>;
+    kernel<<<grid, UNIT_THREADS, smem, stream>>>(
         D.rowptr, static_cast<const uint4*>(colp), static_cast<const uint4*>(valp), D.n_rows, x, D.scale, D.n_cols,
-        vstruct, ts, S, z, grad, F_part, D.unit_groups_max, D.f_ticket, F_out);
+        vstruct, ts, S, z, grad, F_part, D.unit_groups_max, per, D.f_ticket, F_out);
     return cudaGetLastError();
 }
 
@@ -1193,8 +1204,10 @@ int dose_form_effective(const DevCSR& D) {
 
 cudaError_t spmv_configure() {
     cudaError_t e = cudaSuccess;
-    for (const void* k : {(const void*)k_dose_units<false, false>, (const void*)k_dose_units<true, false>,
-                          (const void*)k_dose_units<true, true>, (const void*)k_dose_merge<false, false>,
+    for (const void* k : {(const void*)k_dose_units<false, false, false>, (const void*)k_dose_units<true, false, false>,
+                          (const void*)k_dose_units<true, true, false>, (const void*)k_dose_units<false, false, true>,
+                          (const void*)k_dose_units<true, false, true>,
+                          (const void*)k_dose_units<true, true, true>, (const void*)k_dose_merge<false, false>,
                           (const void*)k_dose_merge<true, false>, (const void*)k_dose_merge<true, true>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, UNITS_SMEM_MAX);
     return e;

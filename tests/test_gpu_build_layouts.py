@@ -24,6 +24,7 @@ def torch():
     (257, [4, 6], [5, 5], 20.0), (515, [9, 8], [9, 8], 60.0),
     (1030, [1] * 300, [2] * 300, 12.0),                 # more beams than shared memory keeps offsets of
     (300, [120, 120], [30, 30], 900.0),                  # 7200 beamlets: two tiles of the placement
+    (77824, [4], [6], 2.0), (77825, [4], [6], 2.0),     # 16 rows to each of the dose's warps, and units of 32 from there
     (550000, [270], [30], 1.0),                         # chunks of more rows than one window
 ])
 def test_layouts_hold_every_entry(torch, V, rows, cols, mean_row):
